@@ -142,7 +142,7 @@ def prepare(case, seed):
     eng.load_layers(0, layers)
     eng.load_head(head)
     kv = clasp.KVCache(ccfg, device=dev)
-    st = {"case": case, "cfg": cfg, "eng": eng, "kv": kv}
+    st = {"case": case, "cfg": cfg, "eng": eng, "kv": kv, "layers": layers, "head": head}
     if kind not in ("prefill", "generate"):
         # a verified context: keys and values as the projections of unit-variance rows give them
         kv.k.normal_(0.0, 1.28, generator=g)
@@ -161,7 +161,7 @@ def prepare(case, seed):
 
     if kind == "search":
         _, hid = eng.verify(tokens, C0, kv, 1)          # [T, L+1, d]: the objective's hidden states
-        st["hidden"] = hid
+        st["hidden"], st["objective"] = hid, tokens
     elif kind == "verify":
         n = case["rows"]
         st["tokens"] = successors(tokens[:1], n - 1)
@@ -299,3 +299,143 @@ def tolerance(case):
     if case["kind"] == "search":
         return {"rel": 1e-2, "max": 6e-2, "differ": 0.0}
     return {"rel": 1.8e-2, "max": 0.12, "differ": 0.0}
+
+
+# ---------------------------------------------------------------- the same results in 64 bits
+# Plain torch on the state's weights, cache and tokens; hidden states of an objective are computed here from its
+# tokens, nothing is taken from the library but whole numbers (drafted tokens).
+
+def _rope64(x, pos, theta):
+    hd = x.shape[-1]
+    inv = theta ** (-torch.arange(0, hd, 2, dtype=torch.float64, device=x.device) / hd)
+    a = pos.double()[:, None, None] * inv
+    lo, hi = x[..., :hd // 2], x[..., hd // 2:]
+    return torch.cat([lo * a.cos() - hi * a.sin(), hi * a.cos() + lo * a.sin()], -1)
+
+
+def _norm64(cfg, x, w):
+    return x * torch.rsqrt((x * x).mean(-1, keepdim=True) + cfg.rms_eps) * w.double()
+
+
+def _layer64(cfg, lw, x, pos, ck, cv, own):
+    """One decoder layer over rows x [n, d] that see the keys ck, values cv and the rows `own` [n, n] says; (y, k, v)."""
+    n, nq, nkv, hd = x.shape[0], cfg.n_q_heads, cfg.n_kv_heads, cfg.head_dim
+    h = _norm64(cfg, x, lw["attn_norm"])
+    q = _rope64((h @ lw["wq"].double().T).view(n, nq, hd), pos, cfg.rope_theta) / math.sqrt(hd)
+    k = _rope64((h @ lw["wk"].double().T).view(n, nkv, hd), pos, cfg.rope_theta)
+    v = (h @ lw["wv"].double().T).view(n, nkv, hd)
+    ks, vs = torch.cat([ck.double(), k]), torch.cat([cv.double(), v])
+    o = torch.empty_like(q)
+    for g in range(nkv):
+        heads = slice(g * (nq // nkv), (g + 1) * (nq // nkv))
+        s = torch.einsum("nhd,cd->hnc", q[:, heads], ks[:, g])
+        s[:, :, ck.shape[0]:].masked_fill_(~own, -math.inf)
+        o[:, heads] = torch.einsum("hnc,cd->nhd", s.softmax(-1), vs[:, g])
+    x = x + o.reshape(n, -1) @ lw["wo"].double().T
+    h = _norm64(cfg, x, lw["mlp_norm"])
+    act = torch.nn.functional.silu(h @ lw["w_gate"].double().T) * (h @ lw["w_up"].double().T)
+    return x + act @ lw["w_down"].double().T, k, v
+
+
+def _forward64(cfg, layers, head, tokens, pos0, ck, cv, skip=None, extra=None):
+    """(hidden [n, L + 1, d], k, v of the rows by layer) of tokens at pos0.. over the cache; `extra`: {layer: (k, v)} after it."""
+    n = tokens.numel()
+    pos = torch.arange(pos0, pos0 + n, device=tokens.device)
+    causal = torch.ones((n, n), dtype=torch.bool, device=tokens.device).tril()
+    x = head["embed"][tokens.long()].double()
+    hid, kv = [x], {}
+    for l in range(cfg.L):
+        if not (skip and skip[l]):
+            k0, v0 = ck[l, :pos0], cv[l, :pos0]
+            if extra and l in extra:
+                m = extra[l][0].shape[0]
+                k0 = torch.cat([k0[:pos0 - m].double(), extra[l][0]])
+                v0 = torch.cat([v0[:pos0 - m].double(), extra[l][1]])
+            x, k, v = _layer64(cfg, layers[l], x, pos, k0, v0, causal)
+            kv[l] = (k, v)
+        hid.append(x)
+    return torch.stack(hid, 1), kv
+
+
+def _logits64(cfg, head, x):
+    h = _norm64(cfg, x, head["final_norm"])
+    return torch.cat([h @ w.double().T for w in head["lm_head"].split(16384)], -1)
+
+
+def _search64(cfg, layers, hid, ck, cv, C0, T, M):
+    L = cfg.L
+    x = hid.transpose(0, 1)                      # [L + 1, T, d]
+    nan = torch.full((L + 1, M + 1), math.nan, dtype=torch.float64, device=x.device)
+    D, margin = nan.clone(), nan.clone()
+    D[:, 0] = 1.0
+
+    def score(i, y):
+        return torch.nn.functional.cosine_similarity(x[i], y, dim=-1, eps=1e-12).mean(-1)
+
+    pos = torch.arange(C0, C0 + T, device=x.device)
+    causal = torch.ones((T, T), dtype=torch.bool, device=x.device).tril()
+    g = {0: x[0]}
+    for i in range(1, L + 1):
+        n = min(i - 1, M)
+        new = {0: x[i]}
+        if n:
+            own = torch.block_diag(*[causal.double()] * n).bool()
+            y, _, _ = _layer64(cfg, layers[i - 1], torch.cat([g[j] for j in range(1, n + 1)]), pos.repeat(n),
+                               ck[i - 1, :C0], cv[i - 1, :C0], own)
+            app = y.view(n, T, -1)
+            skip = torch.stack([g[j - 1] for j in range(1, n + 1)])
+            sa, ss = score(i, app), score(i, skip)
+            take = sa > ss
+            D[i, 1:n + 1], margin[i, 1:n + 1] = torch.where(take, sa, ss), sa - ss
+            for j in range(1, n + 1):
+                new[j] = app[j - 1] if take[j - 1] else skip[j - 1]
+        if i <= M:
+            new[i] = g[i - 1]
+            D[i, i] = score(i, g[i - 1])
+        g = new
+    return {"S": None, "D": D, "margin": margin, "g_final": g[M]}
+
+
+def exact(case, seed):
+    cfg, kind, C0, M, T, K = _shape(case), case["kind"], case["ctx"], case["M"], case["T"], case["K"]
+    st = prepare(case, seed)
+    layers, head, kv = st["layers"], st["head"], st["kv"]
+    ck, cv = kv.k.clone(), kv.v.clone()
+
+    def stack(own):
+        return tuple(torch.stack([own[l][i] for l in range(cfg.L)]) for i in (0, 1))
+
+    if kind == "search":
+        hid, _ = _forward64(cfg, layers, head, st["objective"], C0, ck, cv)
+        return _search64(cfg, layers, hid, ck, cv, C0, T, M)
+    if kind == "verify":
+        hid, own = _forward64(cfg, layers, head, st["tokens"], C0, ck, cv)
+        k, v = stack(own)
+        return {"argmax": None, "hidden": hid, "k": k, "v": v}
+    if kind == "prefill":
+        hid, own = _forward64(cfg, layers, head, st["tokens"], 0, ck, cv)
+        k, v = stack(own)
+        return {"argmax": None, "hidden": hid[-st["hidden"].shape[0]:], "k": k, "v": v}
+    if kind == "generate":
+        tokens = torch.tensor(st["tokens"], device=ck.device)
+        k, v = stack(_forward64(cfg, layers, head, tokens, 0, ck, cv)[1])
+        return {"tokens": None, "hidden": None, "S": None, "k": k, "v": v}
+    if kind == "draft":
+        hid, own = _forward64(cfg, layers, head, st["tokens"], C0, ck, cv, skip=st["mask"])
+        p = _logits64(cfg, head, hid[:, -1]).softmax(-1).max(-1).values
+        for l in range(cfg.L):
+            own.setdefault(l, (ck[l, C0:C0 + 1].double(), cv[l, C0:C0 + 1].double()))
+        k, v = stack(own)
+        return {"token": None, "prob": p, "k": k, "v": v}
+    # a sampled round: the tokens are the library's draws, everything else is computed from them
+    run(st)
+    tokens = st["tokens"].clone()
+    q, extra = [], {}
+    for i in range(K):
+        hid, own = _forward64(cfg, layers, head, tokens[i:i + 1], C0 + i, ck, cv, skip=st["mask"], extra=extra)
+        q.append(_logits64(cfg, head, hid[:, -1]))
+        extra = {l: tuple(torch.cat([extra[l][j], own[l][j]]) if l in extra else own[l][j] for j in (0, 1)) for l in own}
+    hid, own = _forward64(cfg, layers, head, tokens, C0, ck, cv)
+    k, v = stack(own)
+    return {"drafts": None, "q": torch.cat(q), "p": _logits64(cfg, head, hid[:, -1]), "n_acc": None, "committed": None,
+            "hidden": hid, "k": k, "v": v}
