@@ -9,6 +9,7 @@
 
 #include <cstdio>
 #include <cstdlib>
+#include <algorithm>
 #include <array>
 #include <cstring>
 #include <map>
@@ -20,10 +21,12 @@
 #include "kernels.cuh"
 #include "engine2.cuh"
 #include "sampling.cuh"
+#include "wide.cuh"
 
 namespace {
 
 using bf16 = __nv_bfloat16;
+constexpr int WIDE_MIN_ROWS = 128;   // layers over more rows take the products and the attention of wide.cuh
 constexpr int MAX_COUNTERS = 4096;   // tiles of one GEMM launch that may use split-K
 constexpr size_t PARTIAL_FLOATS = (size_t)296 * 2 * 128 * 128 + (1 << 20);
 
@@ -266,6 +269,7 @@ struct GemmCall {
   int64_t ldr = 0;
   void* yo = nullptr;
   int64_t ldo = 0;
+  bool wide = false;         // a decoder layer's product over many rows (gemm_wide)
 };
 
 template <typename TW, int EPI>
@@ -373,8 +377,64 @@ int gemm_tc(clasp_ctx* ctx, const GemmCall& g) {
   return CLASP_OK;
 }
 
+// The operand's tensor map, kept per (buffer, K, box): the workspace's buffers live as long as the context.
+int x_map(clasp_ctx* ctx, const void* x, int K, int rows, int box, CUtensorMap** out) {
+  auto key = std::make_tuple(x, K, rows * 1024 + box);
+  auto it = ctx->xmaps.find(key);
+  if (it == ctx->xmaps.end()) {
+    CUtensorMap mp;
+    if (make_map(ctx, x, rows, K, box, &mp)) return CLASP_ERR_CUDA;
+    it = ctx->xmaps.emplace(key, mp).first;
+  }
+  *out = &it->second;
+  return CLASP_OK;
+}
+
+// Products over more rows than the skinny kernels are made for (wide.cuh).
+int gemm_wide(clasp_ctx* ctx, const GemmCall& g) {
+  namespace wd = clasp::wide;
+  wd::GemmParams p{};
+  p.dual = g.epi == clasp::EPI_SWIGLU ? 1 : 0;
+  const int tn = p.dual ? wd::TN / 2 : wd::TN;
+  p.R = g.R;
+  p.kc = (g.K + wd::BK - 1) / wd::BK;
+  p.n_mats = g.n_mats;
+  p.row_tiles = (g.R + 2 * wd::TM - 1) / (2 * wd::TM);
+  int f_tiles = 0;
+  for (int m = 0; m < g.n_mats; ++m) {
+    p.N[m] = g.N[m];
+    p.f_tiles[m] = (g.N[m] + tn - 1) / tn;
+    p.col_off[m] = g.col_off[m];
+    f_tiles += p.f_tiles[m];
+  }
+  p.tiles = f_tiles * p.row_tiles;
+  // pairs at work: one per two SMs, each with at least a handful of chunks
+  int W = ctx->num_sms / 2;
+  const long long units = (long long)p.tiles * p.kc;
+  if (units / 8 < W) W = units / 8 < 1 ? 1 : (int)(units / 8);
+  // What whole waves of tiles leave over is split over K, together with one whole wave (a tile then has two or three
+  // parts); a last wave that is at least 15/16 full stays whole.
+  const int full = p.tiles / W, left = p.tiles - full * W;
+  p.sk_tiles = left == 0 || (W - left) * 16 <= W ? 0 : left + (full > 0 ? W : 0);
+  if (p.sk_tiles * 2 > MAX_COUNTERS || (size_t)W * 4 * wd::SLOT_FLOATS > PARTIAL_FLOATS) p.sk_tiles = 0;
+  p.epi = g.epi;
+  p.yf = g.yf; p.ldy = g.ldy; p.resid = g.resid; p.ldr = g.ldr; p.yo = (bf16*)g.yo; p.ldo = g.ldo;
+  p.partial = ctx->ws.partial; p.counters = ctx->ws.counters; p.status = ctx->ws.status;
+  p.spin_fast = ctx->wait_limit ? std::min(ctx->wait_limit, clasp::tc::SPIN_FAST) : clasp::tc::SPIN_FAST;
+  p.spin_slow = ctx->wait_limit ? ctx->wait_limit : clasp::tc::SPIN_SLOW;
+  CUtensorMap* mx;
+  int rc = x_map(ctx, g.x, g.K, g.R, wd::TM, &mx);
+  if (rc) return rc;
+  const CUtensorMap* w0 = g.wmap[0];
+  const CUtensorMap* w1 = p.dual ? g.w2map : (g.n_mats > 1 ? g.wmap[1] : w0);
+  const CUtensorMap* w2 = g.n_mats > 2 ? g.wmap[2] : w0;
+  wd::gemm_kernel<<<2 * W, wd::GEMM_THREADS, wd::GEMM_SMEM, ctx->stream>>>(*mx, *w0, *w1, *w2, p);
+  return launch_check(ctx);
+}
+
 int gemm(clasp_ctx* ctx, const GemmCall& g) {
   if (g.R <= 0) return CLASP_OK;
+  if (g.wide) return gemm_wide(ctx, g);
   if (ctx->cfg.dtype == CLASP_FP32) return gemm_simt<float>(ctx, g);
   if (ctx->use_tc) return gemm_tc(ctx, g);
   return gemm_simt<bf16>(ctx, g);
@@ -412,6 +472,36 @@ int attention(clasp_ctx* ctx, int R, int T, int C, const clasp_kv_layer& kv, con
   return launch_check(ctx);
 }
 
+// Attention of many rows on the tensor cores (wide.cuh): own rows' keys and values at own_k / own_v + own_base rows.
+int attention_wide(clasp_ctx* ctx, int R, int T, int C, const clasp_kv_layer& kv, const bf16* own_k, const bf16* own_v,
+                   int64_t own_base) {
+  namespace wd = clasp::wide;
+  const clasp_config& c = ctx->cfg;
+  Workspace& ws = ctx->ws;
+  const int kvd = c.n_kv_heads * c.head_dim, Gq = c.n_q_heads / c.n_kv_heads;
+  wd::AttnParams p{};
+  p.qkv = ws.qkv; p.ldq = (c.n_q_heads + 2 * c.n_kv_heads) * c.head_dim; p.cs = ws.rope;
+  p.C = C; p.R = R; p.T = T; p.nq = c.n_q_heads; p.nkv = c.n_kv_heads;
+  p.blocks = (R * Gq + wd::ATT_PAIRS - 1) / wd::ATT_PAIRS;
+  // few blocks: their key tiles are split so that two CTAs per SM have work (at least four tiles each)
+  const int slots = 2 * ctx->num_sms, items = p.blocks * c.n_kv_heads;
+  const int tiles = (C + R + wd::ATT_TK - 1) / wd::ATT_TK;
+  p.splits = std::max(1, std::min({slots / items, tiles / 4, clasp::ATT_MAX_CACHE_CHUNKS}));
+  p.out = (bf16*)ws.attn; p.part_acc = ws.att_acc; p.part_ml = ws.att_ml; p.status = ws.status;
+  p.spin_fast = ctx->wait_limit ? std::min(ctx->wait_limit, clasp::tc::SPIN_FAST) : clasp::tc::SPIN_FAST;
+  p.spin_slow = ctx->wait_limit ? ctx->wait_limit : clasp::tc::SPIN_SLOW;
+  CUtensorMap mck, mcv, mok, mov;
+  int rc = make_map(ctx, own_k + own_base * kvd, R, kvd, wd::ATT_TK, &mok) | make_map(ctx, own_v + own_base * kvd, R, kvd, wd::ATT_TK, &mov);
+  mck = mok; mcv = mov;
+  if (C > 0) rc |= make_map(ctx, kv.k, C, kvd, wd::ATT_TK, &mck) | make_map(ctx, kv.v, C, kvd, wd::ATT_TK, &mcv);
+  if (rc) return CLASP_ERR_CUDA;
+  wd::attn_kernel<<<items * p.splits, wd::ATT_THREADS, wd::ATT_SMEM, ctx->stream>>>(mck, mcv, mok, mov, p);
+  if ((rc = launch_check(ctx)) || p.splits == 1) return rc;
+  clasp::attn_merge_kernel<bf16, wd::HD><<<R * c.n_q_heads, wd::HD, 0, ctx->stream>>>(ws.att_acc, ws.att_ml, R, c.n_q_heads,
+                                                                                  p.splits, (bf16*)ws.attn);
+  return launch_check(ctx);
+}
+
 template <typename TW>
 int rmsnorm(clasp_ctx* ctx, const float* x, int64_t ldx, const float* w, int R, void* y) {
   clasp::rmsnorm_kernel<TW><<<R, 256, 0, ctx->stream>>>(x, ldx, w, ctx->cfg.d_model, ctx->cfg.rms_eps, (TW*)y);
@@ -437,11 +527,13 @@ int run_layer(clasp_ctx* ctx, int l, const float* x, int64_t ldx, int S, int T, 
   const LayerMaps* mp = tc ? &ctx->maps[l] : nullptr;
   const int R = S * T, d = c.d_model, qd = c.n_q_heads * c.head_dim, kvd = c.n_kv_heads * c.head_dim;
   const int qkvd = qd + 2 * kvd;
+  // more rows than one launch of the skinny product takes: the products are bound by the tensor cores
+  const bool wide = tc && R > WIDE_MIN_ROWS;
   int rc;
   if ((rc = rmsnorm<TW>(ctx, x, ldx, W.attn_norm, R, ws.xn))) return rc;
   {
     GemmCall g;
-    g.x = ws.xn; g.R = R; g.K = d; g.n_mats = 3;
+    g.x = ws.xn; g.R = R; g.K = d; g.n_mats = 3; g.wide = wide;
     g.w[0] = W.wq; g.w[1] = W.wk; g.w[2] = W.wv;
     if (tc) { g.wmap[0] = &mp->wq; g.wmap[1] = &mp->wk; g.wmap[2] = &mp->wv; }
     g.N[0] = qd; g.N[1] = kvd; g.N[2] = kvd;
@@ -455,12 +547,13 @@ int run_layer(clasp_ctx* ctx, int l, const float* x, int64_t ldx, int S, int T, 
   clasp::kv_store_kernel<TW><<<R, 256, 0, ctx->stream>>>(ws.qkv, qkvd, ws.rope, T, c.n_q_heads, c.n_kv_heads,
                                                          c.head_dim, own_k, own_v, own_base);
   if ((rc = launch_check(ctx))) return rc;
-  if (c.head_dim == 128) rc = attention<TW, 128>(ctx, R, T, C, kv, own_k, own_v, own_base);
+  if (wide && c.head_dim == clasp::wide::HD) rc = attention_wide(ctx, R, T, C, kv, (const bf16*)own_k, (const bf16*)own_v, own_base);
+  else if (c.head_dim == 128) rc = attention<TW, 128>(ctx, R, T, C, kv, own_k, own_v, own_base);
   else rc = attention<TW, 64>(ctx, R, T, C, kv, own_k, own_v, own_base);
   if (rc) return rc;
   {
     GemmCall g;
-    g.x = ws.attn; g.R = R; g.K = qd; g.n_mats = 1; g.w[0] = W.wo;
+    g.x = ws.attn; g.R = R; g.K = qd; g.n_mats = 1; g.w[0] = W.wo; g.wide = wide;
     if (tc) g.wmap[0] = &mp->wo;
     g.N[0] = d; g.epi = clasp::EPI_RESID; g.yf = ws.x1; g.ldy = d; g.resid = x; g.ldr = ldx;
     if ((rc = gemm(ctx, g))) return rc;
@@ -468,14 +561,14 @@ int run_layer(clasp_ctx* ctx, int l, const float* x, int64_t ldx, int S, int T, 
   if ((rc = rmsnorm<TW>(ctx, ws.x1, d, W.mlp_norm, R, ws.xn))) return rc;
   {
     GemmCall g;
-    g.x = ws.xn; g.R = R; g.K = d; g.n_mats = 1; g.w[0] = W.w_gate; g.w2 = W.w_up;
+    g.x = ws.xn; g.R = R; g.K = d; g.n_mats = 1; g.w[0] = W.w_gate; g.w2 = W.w_up; g.wide = wide;
     if (tc) { g.wmap[0] = &mp->w_gate; g.w2map = &mp->w_up; }
     g.N[0] = c.d_ffn; g.epi = clasp::EPI_SWIGLU; g.yo = ws.act; g.ldo = c.d_ffn;
     if ((rc = gemm(ctx, g))) return rc;
   }
   {
     GemmCall g;
-    g.x = ws.act; g.R = R; g.K = c.d_ffn; g.n_mats = 1; g.w[0] = W.w_down;
+    g.x = ws.act; g.R = R; g.K = c.d_ffn; g.n_mats = 1; g.w[0] = W.w_down; g.wide = wide;
     if (tc) g.wmap[0] = &mp->w_down;
     g.N[0] = d; g.epi = clasp::EPI_RESID; g.yf = out; g.ldy = ldo; g.resid = ws.x1; g.ldr = d;
     if ((rc = gemm(ctx, g))) return rc;
@@ -946,7 +1039,11 @@ int clasp_create(const clasp_config* cfg, void* workspace, size_t workspace_byte
     }
     ctx->encode = (EncodeTiledFn)fn;
     if (cudaFuncSetAttribute(clasp::tc::gemm_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             220 * 1024) != cudaSuccess) {
+                             220 * 1024) != cudaSuccess ||
+        cudaFuncSetAttribute(clasp::wide::gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, clasp::wide::GEMM_SMEM) !=
+            cudaSuccess ||
+        cudaFuncSetAttribute(clasp::wide::attn_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, clasp::wide::ATT_SMEM) !=
+            cudaSuccess) {
       delete ctx;
       return CLASP_ERR_CUDA;
     }
