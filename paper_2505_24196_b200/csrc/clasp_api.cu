@@ -21,11 +21,13 @@
 #include "kernels.cuh"
 #include "engine2.cuh"
 #include "sampling.cuh"
+#include "small32.cuh"
 #include "wide.cuh"
 
 namespace {
 
 using bf16 = __nv_bfloat16;
+constexpr int S32_MAX_ROWS = 128;    // rows a forward pass of the one-cluster fp32 path takes
 constexpr int WIDE_MIN_ROWS = 128;   // layers over more rows take the products and the attention of wide.cuh
 constexpr int MAX_COUNTERS = 4096;   // tiles of one GEMM launch that may use split-K
 constexpr size_t PARTIAL_FLOATS = (size_t)296 * 2 * 128 * 128 + (1 << 20);
@@ -191,6 +193,9 @@ struct clasp_ctx {
   int cta_cap = 296;
   int smem_budget = 110 * 1024;
   int num_sms = 148;
+  bool use_s32 = false;     // fp32 model that fits one cluster's shared memory: one launch per call (small32.cuh)
+  bool s32_head = false;    // ... and so does its LM head
+  int s32_smem = 0;
   // persistent layer engine
   bool use_engine = false;
   int e_G = 0;              // CTAs of the cooperative grid (one per SM)
@@ -628,6 +633,111 @@ int embed_rows(clasp_ctx* ctx, const int32_t* tokens, int n, float* out, int64_t
 }
 
 
+// ---------------------------------------------------------------- fp32 models of one cluster (small32.cuh)
+namespace s32 = clasp::s32;
+
+const void* s32_kernel(const clasp_config& c) {
+  return c.head_dim == 128 ? (const void*)s32::call_kernel<128> : (const void*)s32::call_kernel<64>;
+}
+
+int s32_launch_config(clasp_ctx* ctx, cudaLaunchConfig_t* lc, cudaLaunchAttribute* attr) {
+  *lc = cudaLaunchConfig_t{};
+  lc->gridDim = dim3(s32::CTAS);
+  lc->blockDim = dim3(s32::THREADS);
+  lc->dynamicSmemBytes = ctx->s32_smem;
+  lc->stream = ctx->stream;
+  attr->id = cudaLaunchAttributeClusterDimension;
+  attr->val.clusterDim.x = s32::CTAS; attr->val.clusterDim.y = 1; attr->val.clusterDim.z = 1;
+  lc->attrs = attr;
+  lc->numAttrs = 1;
+  return CLASP_OK;
+}
+
+// The model takes the one-launch path when every CTA's slices of a layer fit its shared memory beside the rows of a pass
+// and a warp has at most MAX_F features of a product.  Anything larger keeps one kernel per step.
+int s32_setup(clasp_ctx* ctx) {
+  const clasp_config& c = ctx->cfg;
+  ctx->use_s32 = ctx->s32_head = false;
+  if (c.dtype != CLASP_FP32 || (c.flags & (CLASP_FLAG_MULTI_KERNEL | CLASP_FLAG_PRUNE))) return CLASP_OK;
+  const int d = c.d_model, qd = c.n_q_heads * c.head_dim, kvd = c.n_kv_heads * c.head_dim, cap = s32::MAX_F * s32::WARPS;
+  if (c.L > s32::MAX_L || c.max_M + 1 > s32::MAX_STATES || s32::slice_cap(qd + 2 * kvd) > cap || s32::slice_cap(d) > cap ||
+      2 * s32::slice_cap(c.d_ffn) > cap)
+    return CLASP_OK;
+  int dev = 0, optin = 0;
+  CUDA_TRY(cudaGetDevice(&dev));
+  CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+  const long long bytes = 4LL * s32::smem_floats(d, qd, kvd, c.d_ffn, c.head_dim, c.L, c.max_M);
+  const void* k = s32_kernel(c);
+  cudaFuncAttributes fa;
+  CUDA_TRY(cudaFuncGetAttributes(&fa, k));
+  if (bytes + (long long)fa.sharedSizeBytes > optin) return CLASP_OK;
+  CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+  CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  ctx->s32_smem = (int)bytes;
+  cudaLaunchConfig_t lc;
+  cudaLaunchAttribute attr;
+  s32_launch_config(ctx, &lc, &attr);
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, k, &lc) != cudaSuccess || n < 1) {
+    cudaGetLastError();   // (a device that cannot place such a cluster: one kernel per step)
+    return CLASP_OK;
+  }
+  ctx->use_s32 = true;
+  ctx->s32_head = s32::slice_cap(c.vocab) <= 2 * s32::slice_cap(c.d_ffn);
+  return CLASP_OK;
+}
+
+void s32_params(clasp_ctx* ctx, s32::Params* p, int T, int C, int pos0) {
+  const clasp_config& c = ctx->cfg;
+  Workspace& ws = ctx->ws;
+  memset(p, 0, sizeof(*p));
+  p->d = c.d_model; p->qd = c.n_q_heads * c.head_dim; p->kvd = c.n_kv_heads * c.head_dim;
+  p->nq = c.n_q_heads; p->nkv = c.n_kv_heads; p->dffn = c.d_ffn; p->vocab = c.vocab;
+  p->eps = c.rms_eps; p->theta = (double)c.rope_theta;
+  p->T = T; p->C = C; p->pos0 = pos0;
+  p->qkv = ws.qkv; p->attn = (float*)ws.attn; p->x1 = ws.x1; p->act = (float*)ws.act; p->logits = ws.logits; p->rope = ws.rope;
+  p->status = ws.status;
+  p->spin_fast = ctx->wait_limit ? std::min(ctx->wait_limit, clasp::tc::SPIN_FAST) : clasp::tc::SPIN_FAST;
+  p->spin_slow = ctx->wait_limit ? ctx->wait_limit : clasp::tc::SPIN_SLOW;
+}
+
+void s32_layer(clasp_ctx* ctx, s32::Params* p, int l, const clasp_kv_layer& kv) {
+  const clasp_layer_weights& w = ctx->layers[l];
+  s32::LayerPtrs& q = p->layer[p->n_layers++];
+  q.attn_norm = w.attn_norm; q.mlp_norm = w.mlp_norm;
+  q.wq = (const float*)w.wq; q.wk = (const float*)w.wk; q.wv = (const float*)w.wv; q.wo = (const float*)w.wo;
+  q.wg = (const float*)w.w_gate; q.wu = (const float*)w.w_up; q.wd = (const float*)w.w_down;
+  q.ck = (float*)kv.k; q.cv = (float*)kv.v;
+}
+
+int s32_launch(clasp_ctx* ctx, s32::Params* p) {
+  cudaLaunchConfig_t lc;
+  cudaLaunchAttribute attr;
+  s32_launch_config(ctx, &lc, &attr);
+  void* args[] = {(void*)p};
+  if (cudaLaunchKernelExC(&lc, s32_kernel(ctx->cfg), args) != cudaSuccess) return CLASP_ERR_CUDA;
+  return launch_check(ctx);
+}
+
+// n tokens at position pos0 through the layers added to *p, then the head over the last n_head rows
+int s32_forward(clasp_ctx* ctx, s32::Params* p, const int32_t* tokens, int n, float* hidden_out, int n_head, int32_t* argmax_out,
+                float* top1, float* logits_out) {
+  const clasp_config& c = ctx->cfg;
+  p->tokens = tokens; p->embed = (const float*)ctx->embed;
+  if (hidden_out) {
+    p->x_base[0] = hidden_out; p->x_step = c.d_model; p->ldx = (int64_t)(c.L + 1) * c.d_model;
+  } else {
+    p->x_base[0] = ctx->ws.hping; p->x_base[1] = ctx->ws.hpong; p->ldx = c.d_model;
+  }
+  p->final_norm = ctx->final_norm; p->lm_head = (const float*)ctx->lm_head;
+  p->argmax_out = argmax_out; p->top1_out = top1; p->logits_out = logits_out;
+  p->head_rows = ctx->s32_head ? n_head : 0;
+  int rc = s32_launch(ctx, p);
+  if (rc || n_head == 0 || ctx->s32_head) return rc;
+  const float* x = p->x_step > 0 ? p->x_base[0] + p->n_layers * p->x_step : p->x_base[p->n_layers & 1];
+  return run_head(ctx, x + (int64_t)(n - n_head) * p->ldx, p->ldx, n_head, argmax_out, top1, logits_out);
+}
+
 // ---------------------------------------------------------------- persistent layer engine
 // Host side of engine2.cuh: builds the job list of a call and launches the cooperative
 // kernel once.  Used by the bf16 tensor-core configuration; the per-kernel sequences
@@ -1054,6 +1164,10 @@ int clasp_create(const clasp_config* cfg, void* workspace, size_t workspace_byte
     delete ctx;
     return CLASP_ERR_CUDA;
   }
+  if (s32_setup(ctx) != CLASP_OK) {
+    delete ctx;
+    return CLASP_ERR_CUDA;
+  }
   if (ctx->use_tc) {
     if (engine_setup(ctx) != CLASP_OK || cudaMemsetAsync(ws.ctl, 0, 256, ctx->stream) != cudaSuccess ||
         cudaMemsetAsync(ws.e_att_acc, 0, ws.e_att_bytes, ctx->stream) != cudaSuccess) {
@@ -1162,6 +1276,15 @@ int clasp_dp_search(clasp_ctx* ctx, const float* hidden_states, int64_t layer_st
     return CLASP_ERR_INVALID_ARG;
   if (M > 0 && !layers_ready(ctx)) return CLASP_ERR_NOT_LOADED;
   Workspace& ws = ctx->ws;
+  if (ctx->use_s32 && M > 0 && T <= s32::ROW_COS) {
+    s32::Params p;
+    s32_params(ctx, &p, T, ctx_len, pos0);
+    for (int l = 0; l < L; ++l) s32_layer(ctx, &p, l, kv[l]);
+    p.search = 1; p.hidden = hidden_states; p.layer_stride = layer_stride; p.token_stride = token_stride; p.M = M;
+    p.G = ws.G; p.g[0] = ws.grow[0]; p.g[1] = ws.grow[1];
+    p.scores = scores; p.margins = margins; p.g_final = g_final; p.forced = forced_choice; p.skip_mask = skip_mask;
+    return s32_launch(ctx, &p);
+  }
   const int ncell = (L + 1) * (M + 1);
   clasp::fill_tables_kernel<<<(ncell + 255) / 256, 256, 0, ctx->stream>>>(scores, margins, ws.choice, ncell);
   int rc = launch_check(ctx);
@@ -1285,6 +1408,12 @@ int verify_impl(clasp_ctx* ctx, const int32_t* tokens, int32_t n, int32_t pos0, 
   if (!layers_ready(ctx) || !ctx->embed) return CLASP_ERR_NOT_LOADED;
   const int d = c.d_model, L = c.L;
   int rc;
+  if (ctx->use_s32 && n <= S32_MAX_ROWS) {
+    s32::Params p;
+    s32_params(ctx, &p, n, pos0, pos0);
+    for (int l = 0; l < L; ++l) s32_layer(ctx, &p, l, kv[l]);
+    return s32_forward(ctx, &p, tokens, n, hidden_out, n_head_rows, argmax_out, nullptr, logits_out);
+  }
   if ((rc = rope_table(ctx, n, pos0))) return rc;
   if (ctx->use_engine && n <= pk::MAX_ROWS) {
     // embedding gather, then every layer and the head in one cooperative launch
@@ -1354,6 +1483,13 @@ int draft_impl(clasp_ctx* ctx, const uint8_t* skip_mask_host, const int32_t* tok
     if (!skip_mask_host[l] && (!kv[l].k || !kv[l].v || !kv_aligned(kv + l, 1))) return CLASP_ERR_INVALID_ARG;
   const int d = c.d_model;
   int rc;
+  if (ctx->use_s32) {
+    s32::Params p;
+    s32_params(ctx, &p, 1, pos, pos);
+    for (int l = 0; l < c.L; ++l)
+      if (!skip_mask_host[l]) s32_layer(ctx, &p, l, kv[l]);
+    return s32_forward(ctx, &p, token_in, 1, nullptr, 1, token_out, top1_prob_out, logits_out);
+  }
   if ((rc = rope_table(ctx, 1, pos))) return rc;
   float* a = ctx->ws.hping;
   float* b = ctx->ws.hpong;
