@@ -663,24 +663,36 @@ int s32_setup(clasp_ctx* ctx) {
   if (c.L > s32::MAX_L || c.max_M + 1 > s32::MAX_STATES || s32::slice_cap(qd + 2 * kvd) > cap || s32::slice_cap(d) > cap ||
       2 * s32::slice_cap(c.d_ffn) > cap)
     return CLASP_OK;
-  int dev = 0, optin = 0;
+  // whether a device can place the cluster at all is asked once per device (the question takes milliseconds)
+  static std::mutex mutex;
+  static int limit[2][64];   // [head dimension 128][device]: usable dynamic shared memory, -1: no, 0: not asked yet
+  int dev = 0;
   CUDA_TRY(cudaGetDevice(&dev));
-  CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-  const long long bytes = 4LL * s32::smem_floats(d, qd, kvd, c.d_ffn, c.head_dim, c.L, c.max_M);
+  if (dev >= 64) return CLASP_OK;
   const void* k = s32_kernel(c);
-  cudaFuncAttributes fa;
-  CUDA_TRY(cudaFuncGetAttributes(&fa, k));
-  if (bytes + (long long)fa.sharedSizeBytes > optin) return CLASP_OK;
-  CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-  CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-  ctx->s32_smem = (int)bytes;
-  cudaLaunchConfig_t lc;
-  cudaLaunchAttribute attr;
-  s32_launch_config(ctx, &lc, &attr);
-  int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, k, &lc) != cudaSuccess || n < 1) {
-    cudaGetLastError();   // (a device that cannot place such a cluster: one kernel per step)
-    return CLASP_OK;
+  {
+    std::lock_guard<std::mutex> lock(mutex);
+    int& lim = limit[c.head_dim == 128][dev];
+    if (lim == 0) {
+      int optin = 0;
+      cudaFuncAttributes fa;
+      CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+      CUDA_TRY(cudaFuncGetAttributes(&fa, k));
+      const int dyn = optin - (int)fa.sharedSizeBytes;
+      CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
+      CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+      ctx->s32_smem = dyn;
+      cudaLaunchConfig_t lc;
+      cudaLaunchAttribute attr;
+      s32_launch_config(ctx, &lc, &attr);
+      int n = 0;
+      const bool ok = cudaOccupancyMaxActiveClusters(&n, k, &lc) == cudaSuccess && n > 0;
+      if (!ok) cudaGetLastError();   // (such a device keeps one kernel per step)
+      lim = ok ? dyn : -1;
+    }
+    const long long bytes = 4LL * s32::smem_floats(d, qd, kvd, c.d_ffn, c.head_dim, c.L, c.max_M);
+    if (lim < 0 || bytes > lim) return CLASP_OK;
+    ctx->s32_smem = (int)bytes;
   }
   ctx->use_s32 = true;
   ctx->s32_head = s32::slice_cap(c.vocab) <= 2 * s32::slice_cap(c.d_ffn);
@@ -894,7 +906,8 @@ double job_bytes(const clasp_ctx* ctx, const pk::Job& J) {
 
 // Launch the engine over ctx->e_jobs.  Rmax: most rows of any job; head_off: first row of the
 // previous job that the head job (if any) reads.
-int engine_launch(clasp_ctx* ctx, int Rmax, int head_off, int search_ctx = -1) {
+// `setup`: rotary table and the call's own tables or embedded rows; the rest of it is filled in here.
+int engine_launch(clasp_ctx* ctx, int Rmax, int head_off, clasp::SetupArgs setup, int search_ctx = -1) {
   const clasp_config& c = ctx->cfg;
   Workspace& ws = ctx->ws;
   if (ctx->e_jobs.empty()) return CLASP_OK;
@@ -994,9 +1007,14 @@ int engine_launch(clasp_ctx* ctx, int Rmax, int head_off, int search_ctx = -1) {
   }
   CUDA_TRY(cudaMemcpyAsync(ws.jobs, ctx->e_jobs.data(), ctx->e_jobs.size() * sizeof(pk::Job),
                            cudaMemcpyHostToDevice, ctx->stream));
-  CUDA_TRY(cudaMemsetAsync(ws.ctl, 0, 4, ctx->stream));  // abort flag; the status word is sticky
-  CUDA_TRY(cudaMemsetAsync(ws.ss_a, 0, ws.acc_bytes, ctx->stream));  // all fixed-point accumulators
-  CUDA_TRY(cudaMemsetAsync(ws.flags, 0, (size_t)pk::N_FLAGS * (ctx->e_G + 32) * sizeof(int), ctx->stream));
+  setup.abort = &ws.ctl->abort;   // (the status word is sticky)
+  setup.zero = (uint4*)ws.ss_a; setup.n_zero = (int)(ws.acc_bytes / 16);   // all fixed-point accumulators
+  setup.flags = ws.flags; setup.n_flags = pk::N_FLAGS * (ctx->e_G + 32);
+  clasp::setup_kernel<<<ctx->e_G, 256, 0, ctx->stream>>>(setup);
+  {
+    const int rc = launch_check(ctx);
+    if (rc) return rc;
+  }
 
   pk::Params P{};
   P.c.L = c.L; P.c.d = d; P.c.qd = qd; P.c.kvd = c.n_kv_heads * c.head_dim; P.c.hd = c.head_dim;
@@ -1079,6 +1097,16 @@ int engine_launch(clasp_ctx* ctx, int Rmax, int head_off, int search_ctx = -1) {
   }
   ctx->launches += 1;
   return err == cudaSuccess ? CLASP_OK : CLASP_ERR_CUDA;
+}
+
+clasp::SetupArgs setup_args(const clasp_ctx* ctx, int T, int pos0) {
+  clasp::SetupArgs a{};
+  a.cs = ctx->ws.rope; a.T = T; a.half = ctx->cfg.head_dim / 2; a.pos0 = pos0; a.theta = (double)ctx->cfg.rope_theta;
+  return a;
+}
+void setup_tokens(const clasp_ctx* ctx, clasp::SetupArgs* a, const int32_t* tokens, int n, float* out, int64_t ldo) {
+  a->tokens = tokens; a->table = (const bf16*)ctx->embed; a->n_tokens = n; a->d = ctx->cfg.d_model; a->vocab = ctx->cfg.vocab;
+  a->out = out; a->ldo = ldo;
 }
 
 // a decoder-layer job with the fields every caller sets the same way
@@ -1264,15 +1292,15 @@ int clasp_layer_forward(clasp_ctx* ctx, int32_t layer, const float* x_in, int64_
   if ((int64_t)S * T > ctx->cfg.max_rows || ctx_len > ctx->cfg.max_ctx || pos0 + T > ctx->cfg.max_ctx)
     return CLASP_ERR_CAPACITY;
   if (!ctx->loaded[layer]) return CLASP_ERR_NOT_LOADED;
-  int rc = rope_table(ctx, T, pos0);
-  if (rc) return rc;
   if (ctx->use_engine && S * T <= pk::MAX_ROWS && (!write_kv || pos0 == ctx_len)) {
     pk::Job J = layer_job(ctx, layer, S, T, ctx_len, write_kv != 0, *kv_layer);
     J.prep = 1; J.x_in = x_in; J.ldx = in_stride; J.x_out = x_out; J.ldo = out_stride;
     ctx->e_jobs.assign(1, J);
     link_jobs(ctx->e_jobs);
-    return engine_launch(ctx, S * T, 0);
+    return engine_launch(ctx, S * T, 0, setup_args(ctx, T, pos0));
   }
+  int rc = rope_table(ctx, T, pos0);
+  if (rc) return rc;
   return run_layer_any(ctx, layer, x_in, in_stride, S, T, ctx_len, pos0, *kv_layer, write_kv != 0, x_out,
                        out_stride);
 }
@@ -1304,17 +1332,12 @@ int clasp_dp_search(clasp_ctx* ctx, const float* hidden_states, int64_t layer_st
     return s32_launch(ctx, &p);
   }
   const int ncell = (L + 1) * (M + 1);
-  clasp::fill_tables_kernel<<<(ncell + 255) / 256, 256, 0, ctx->stream>>>(scores, margins, ws.choice, ncell);
-  int rc = launch_check(ctx);
-  if (rc) return rc;
-  if ((rc = rope_table(ctx, T, pos0))) return rc;
+  int rc;
   const int64_t Td = (int64_t)T * d;
   const bool prune = (c.flags & CLASP_FLAG_PRUNE) != 0;
   if (ctx->use_engine && M > 0 && M * T <= pk::MAX_ROWS) {
     // one cooperative launch for the whole search: step i = (layer i-1 over the candidate
     // states) + (Eq. 2 select); row 0 of the g table is x_i itself and is never stored
-    clasp::dp_origin_kernel<<<1, 32, 0, ctx->stream>>>(scores, ws.choice);
-    if ((rc = launch_check(ctx))) return rc;
     ctx->e_jobs.clear();
     int cur = 0, prev_lo = 1;
     for (int i = 1; i <= L; ++i) {
@@ -1361,10 +1384,15 @@ int clasp_dp_search(clasp_ctx* ctx, const float* hidden_states, int64_t layer_st
           ctx->e_jobs[k + 1].dual_src = 1;
         }
     link_jobs(ctx->e_jobs);
-    if ((rc = engine_launch(ctx, M * T, 0, ctx_len))) return rc;
+    clasp::SetupArgs setup = setup_args(ctx, T, pos0);
+    setup.D = scores; setup.margin = margins; setup.choice = ws.choice; setup.n_cells = ncell;
+    if ((rc = engine_launch(ctx, M * T, 0, setup, ctx_len))) return rc;
     clasp::backtrack_kernel<<<1, 32, 0, ctx->stream>>>(ws.choice, L, M, skip_mask);
     return launch_check(ctx);
   }
+  clasp::fill_tables_kernel<<<(ncell + 255) / 256, 256, 0, ctx->stream>>>(scores, margins, ws.choice, ncell);
+  if ((rc = launch_check(ctx))) return rc;
+  if ((rc = rope_table(ctx, T, pos0))) return rc;
   {
     clasp::DpStepArgs a0{};  // g[0][0] = x_0, D[0][0] = 1: the b == 0 path of a step over x_0 itself
     a0.x_i = hidden_states; a0.x_tok_stride = token_stride; a0.G = ws.G; a0.g_prev = ws.grow[0];
@@ -1432,12 +1460,12 @@ int verify_impl(clasp_ctx* ctx, const int32_t* tokens, int32_t n, int32_t pos0, 
     for (int l = 0; l < L; ++l) s32_layer(ctx, &p, l, kv[l]);
     return s32_forward(ctx, &p, tokens, n, hidden_out, n_head_rows, argmax_out, nullptr, logits_out);
   }
-  if ((rc = rope_table(ctx, n, pos0))) return rc;
   if (ctx->use_engine && n <= pk::MAX_ROWS) {
     // embedding gather, then every layer and the head in one cooperative launch
     float* h0 = hidden_out ? hidden_out : ctx->ws.hping;
     const int64_t ld = hidden_out ? (int64_t)(L + 1) * d : d;
-    if ((rc = embed_rows(ctx, tokens, n, h0, ld))) return rc;
+    clasp::SetupArgs setup = setup_args(ctx, n, pos0);
+    setup_tokens(ctx, &setup, tokens, n, h0, ld);
     ctx->e_jobs.clear();
     float* a = ctx->ws.hping;
     float* b = ctx->ws.hpong;
@@ -1461,8 +1489,9 @@ int verify_impl(clasp_ctx* ctx, const int32_t* tokens, int32_t n, int32_t pos0, 
       ctx->e_jobs.push_back(H);
     }
     link_jobs(ctx->e_jobs);
-    return engine_launch(ctx, n, n_head_rows > 0 ? n - n_head_rows : 0);
+    return engine_launch(ctx, n, n_head_rows > 0 ? n - n_head_rows : 0, setup);
   }
+  if ((rc = rope_table(ctx, n, pos0))) return rc;
   const float* x;
   int64_t ldx;
   if (hidden_out) {
@@ -1508,13 +1537,13 @@ int draft_impl(clasp_ctx* ctx, const uint8_t* skip_mask_host, const int32_t* tok
       if (!skip_mask_host[l]) s32_layer(ctx, &p, l, kv[l]);
     return s32_forward(ctx, &p, token_in, 1, nullptr, 1, token_out, top1_prob_out, logits_out);
   }
-  if ((rc = rope_table(ctx, 1, pos))) return rc;
   float* a = ctx->ws.hping;
   float* b = ctx->ws.hpong;
-  if ((rc = embed_rows(ctx, token_in, 1, a, d))) return rc;
   int n_kept = 0;
   for (int l = 0; l < c.L; ++l) n_kept += skip_mask_host[l] ? 0 : 1;
   if (ctx->use_engine && n_kept > 0) {
+    clasp::SetupArgs setup = setup_args(ctx, 1, pos);
+    setup_tokens(ctx, &setup, token_in, 1, a, d);
     ctx->e_jobs.clear();
     for (int l = 0; l < c.L; ++l) {
       if (skip_mask_host[l]) continue;  // skipped layer: nothing read, nothing written
@@ -1533,8 +1562,10 @@ int draft_impl(clasp_ctx* ctx, const uint8_t* skip_mask_host, const int32_t* tok
     H.logits_out = logits_out;
     ctx->e_jobs.push_back(H);
     link_jobs(ctx->e_jobs);
-    return engine_launch(ctx, 1, 0);
+    return engine_launch(ctx, 1, 0, setup);
   }
+  if ((rc = rope_table(ctx, 1, pos))) return rc;
+  if ((rc = embed_rows(ctx, token_in, 1, a, d))) return rc;
   for (int l = 0; l < c.L; ++l) {
     if (skip_mask_host[l]) continue;  // skipped layer: state passes through, nothing read or written
     if (!kv[l].k || !kv[l].v) return CLASP_ERR_INVALID_ARG;

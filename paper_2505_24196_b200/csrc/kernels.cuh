@@ -146,14 +146,17 @@ __global__ void gemm_simt_kernel(const TW* __restrict__ x, int64_t ldx, const TW
 // ---------------------------------------------------------------- rotary table
 // cs[t, i] = (cos, sin) of (pos0 + t) * theta^(-2i/hd), evaluated in double so
 // that long contexts do not lose the angle's low bits.
-__global__ void rope_table_kernel(float2* __restrict__ cs, int T, int half, int pos0, double theta) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= T * half) return;
+__device__ __forceinline__ float2 rope_entry(int idx, int half, int pos0, double theta) {
   const int t = idx / half, i = idx % half;
   const double inv = exp2(-(2.0 * i / (2.0 * half)) * log2(theta));
   double s, c;
   sincos((double)(pos0 + t) * inv, &s, &c);
-  cs[idx] = make_float2((float)c, (float)s);
+  return make_float2((float)c, (float)s);
+}
+__global__ void rope_table_kernel(float2* __restrict__ cs, int T, int half, int pos0, double theta) {
+  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= T * half) return;
+  cs[idx] = rope_entry(idx, half, pos0, theta);
 }
 
 // K/V of the rows: rotate k, round k and v to the cache dtype and store them at row
@@ -510,14 +513,6 @@ __global__ void fill_tables_kernel(float* D, float* margin, uint8_t* choice, int
   choice[idx] = 255;
 }
 
-// D(0, 0) = 1 and its choice entry: the origin of the table (g[0][0] = x_0)
-__global__ void dp_origin_kernel(float* D, uint8_t* choice) {
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    D[0] = 1.0f;
-    choice[0] = 0;
-  }
-}
-
 // rows of floats: dst[r, :] = src[r, :] (strided)
 __global__ void copy_rows_kernel(const float* __restrict__ src, int64_t lds, float* __restrict__ dst,
                                  int64_t ldd, int d) {
@@ -581,6 +576,58 @@ __global__ void argmax_kernel(const float* __restrict__ logits, int vocab, int32
     for (int w2 = 0; w2 < nw; ++w2) tot += sv[w2];
     top1_prob[r] = 1.0f / tot;
   }
+}
+
+// ---------------------------------------------------------------- set-up of a launch of the persistent kernel
+// Everything that kernel expects to find: the rotary table, a search's empty tables (origin set) or a forward pass's
+// embedded rows, zeroed accumulators, flags and abort word.  One launch: as six operations on the stream (four kernels'
+// worth of ramps, three memsets) they took longer than a layer of a small model.
+struct SetupArgs {
+  float2* cs;            // rotary table
+  int T, half, pos0;
+  double theta;
+  float* D;              // search: tables of n_cells cells (n_cells == 0: none)
+  float* margin;
+  uint8_t* choice;
+  int n_cells;
+  const int32_t* tokens; // forward: n_tokens rows of the table into out
+  const __nv_bfloat16* table;
+  int n_tokens, d, vocab;
+  float* out;
+  int64_t ldo;
+  uint4* zero;           // n_zero 16-byte pieces
+  int n_zero;
+  int* flags;
+  int n_flags;
+  int* abort;
+};
+
+__global__ void __launch_bounds__(256) setup_kernel(const SetupArgs a) {
+  const int tid = blockIdx.x * blockDim.x + threadIdx.x, n = gridDim.x * blockDim.x;
+  // (the rotary table first: its double arithmetic is the longest chain; from the last block downwards, where the other
+  // jobs have least to do)
+  for (int k = n - 1 - tid; k < a.T * a.half; k += n) a.cs[k] = rope_entry(k, a.half, a.pos0, a.theta);
+  for (int r = blockIdx.x; r < a.n_tokens; r += gridDim.x) {
+    int tok = a.tokens[r];
+    tok = tok < 0 ? 0 : (tok >= a.vocab ? a.vocab - 1 : tok);
+    const __nv_bfloat16* src = a.table + (int64_t)tok * a.d;
+    for (int c = threadIdx.x * 8; c < a.d; c += blockDim.x * 8) {
+      float f[8];
+      load8(src + c, f);
+      float4* dst = reinterpret_cast<float4*>(a.out + r * a.ldo + c);
+      dst[0] = make_float4(f[0], f[1], f[2], f[3]);
+      dst[1] = make_float4(f[4], f[5], f[6], f[7]);
+    }
+  }
+  for (int k = tid; k < a.n_cells; k += n) {
+    const float v = k == 0 ? 1.0f : __int_as_float(0x7fc00000);   // D(0, 0) = 1 (g[0][0] = x_0)
+    a.D[k] = v;
+    if (a.margin) a.margin[k] = __int_as_float(0x7fc00000);
+    a.choice[k] = k == 0 ? 0 : 255;
+  }
+  for (int k = tid; k < a.n_zero; k += n) a.zero[k] = make_uint4(0, 0, 0, 0);
+  for (int k = tid; k < a.n_flags; k += n) a.flags[k] = 0;
+  if (tid == 0) *a.abort = 0;
 }
 
 }  // namespace clasp
