@@ -90,9 +90,10 @@ typedef struct clasp_config {
                                    reached, j < M - (L - i): Algorithm 1 computes them, but the backtrack
                                    can never visit them.  Skip mask, g[L][M] and every reachable cell are
                                    unchanged; the cells left out read NaN in `scores` and `margins`. */
-#define CLASP_FLAG_MULTI_KERNEL 4 /* diagnostics, bf16 model: one kernel per step (tcgen05
-                                   GEMM, attention, norm, Eq. 2 select ...) instead of the
-                                   persistent kernel that runs a whole call in one launch */
+#define CLASP_FLAG_MULTI_KERNEL 4 /* diagnostics: one kernel per step (GEMM, attention, norm,
+                                   Eq. 2 select ...) instead of the persistent kernel (bf16) or
+                                   the one-cluster kernel (small fp32 models) that runs a whole
+                                   call in one launch */
 
 #define CLASP_FLAG_NO_ATT_TC 16 /* diagnostics: searches over long contexts (about 4000 visible positions or
                                    more; 2500 when a kv head serves at most 64 (row, query head) pairs, 1000

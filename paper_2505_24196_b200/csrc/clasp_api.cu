@@ -27,7 +27,13 @@
 namespace {
 
 using bf16 = __nv_bfloat16;
-constexpr int S32_MAX_ROWS = 128;    // rows a forward pass of the one-cluster fp32 path takes
+// Calls of the one-cluster fp32 path: its 16 SMs lose the attention to the whole chip when rows and positions are many.
+// Measured on the small fp32 model, one launch against one kernel per step, us: 1 row at 64 / 1000 / 4000 positions 140 /
+// 404, 233 / 413, 555 / 462; 16 rows at 500 506 / 709; 32 rows at 1000 1368 / 1095; 64 rows at 0 / 500 946 / 1708, 1957 /
+// 1707; 128 rows at 0 / 500 2360 / 2957, 4037 / 2965; searches of 16 rows at 1000 524 / 650, 32 rows at 500 / 1500
+// 704 / 943, 1248 / 1028.
+constexpr int S32_MAX_ROWS = 128, S32_MAX_KEYS = 2048;
+constexpr long long S32_MAX_SCORES = 65536;   // rows x query heads x keys
 constexpr int WIDE_MIN_ROWS = 128;   // layers over more rows take the products and the attention of wide.cuh
 constexpr int MAX_COUNTERS = 4096;   // tiles of one GEMM launch that may use split-K
 constexpr size_t PARTIAL_FLOATS = (size_t)296 * 2 * 128 * 128 + (1 << 20);
@@ -722,6 +728,11 @@ void s32_layer(clasp_ctx* ctx, s32::Params* p, int l, const clasp_kv_layer& kv) 
   q.ck = (float*)kv.k; q.cv = (float*)kv.v;
 }
 
+bool s32_takes(const clasp_ctx* ctx, int rows, int keys) {
+  return ctx->use_s32 && rows <= S32_MAX_ROWS && keys <= S32_MAX_KEYS &&
+         (long long)rows * ctx->cfg.n_q_heads * keys <= S32_MAX_SCORES;
+}
+
 int s32_launch(clasp_ctx* ctx, s32::Params* p) {
   cudaLaunchConfig_t lc;
   cudaLaunchAttribute attr;
@@ -1322,7 +1333,7 @@ int clasp_dp_search(clasp_ctx* ctx, const float* hidden_states, int64_t layer_st
     return CLASP_ERR_INVALID_ARG;
   if (M > 0 && !layers_ready(ctx)) return CLASP_ERR_NOT_LOADED;
   Workspace& ws = ctx->ws;
-  if (ctx->use_s32 && M > 0 && T <= s32::ROW_COS) {
+  if (M > 0 && T <= s32::ROW_COS && s32_takes(ctx, M * T, ctx_len + T)) {
     s32::Params p;
     s32_params(ctx, &p, T, ctx_len, pos0);
     for (int l = 0; l < L; ++l) s32_layer(ctx, &p, l, kv[l]);
@@ -1454,7 +1465,7 @@ int verify_impl(clasp_ctx* ctx, const int32_t* tokens, int32_t n, int32_t pos0, 
   if (!layers_ready(ctx) || !ctx->embed) return CLASP_ERR_NOT_LOADED;
   const int d = c.d_model, L = c.L;
   int rc;
-  if (ctx->use_s32 && n <= S32_MAX_ROWS) {
+  if (s32_takes(ctx, n, pos0 + n)) {
     s32::Params p;
     s32_params(ctx, &p, n, pos0, pos0);
     for (int l = 0; l < L; ++l) s32_layer(ctx, &p, l, kv[l]);
@@ -1530,7 +1541,7 @@ int draft_impl(clasp_ctx* ctx, const uint8_t* skip_mask_host, const int32_t* tok
     if (!skip_mask_host[l] && (!kv[l].k || !kv[l].v || !kv_aligned(kv + l, 1))) return CLASP_ERR_INVALID_ARG;
   const int d = c.d_model;
   int rc;
-  if (ctx->use_s32) {
+  if (s32_takes(ctx, 1, pos + 1)) {
     s32::Params p;
     s32_params(ctx, &p, 1, pos, pos);
     for (int l = 0; l < c.L; ++l)

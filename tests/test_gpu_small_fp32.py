@@ -1,0 +1,107 @@
+"""The one-launch path of fp32 models that fit a cluster (csrc/small32.cuh) against one kernel per step
+(CLASP_FLAG_MULTI_KERNEL, itself compared with the oracle in test_gpu_parity.py): both head dimensions, widths that are no
+multiple of a warp's stride, rows around the passes of eight, ragged key blocks, an LM head that fits its slice and one
+that does not, a draft that skips every layer.
+
+Both sides sum at most 704 products in fp32 in different orders: the expected difference is about sqrt(704) * 6e-8 = 2e-6
+of a value's scale, growing over the layers; 2e-5 leaves a factor of ten."""
+import dataclasses
+
+import pytest
+import torch
+
+import datagen
+import paper_2505_24196_b200 as clasp
+from tests.util import rel_l2
+
+pytestmark = pytest.mark.gpu
+TOL = 2e-5
+TINY = datagen.CONFIGS["tiny"]
+MODELS = {
+    "hd64": TINY,
+    "hd128": dataclasses.replace(TINY, name="hd128", L=5, d_model=192, n_q_heads=2, n_kv_heads=1, head_dim=128, d_ffn=520,
+                                 vocab=1000),
+    "big-head": dataclasses.replace(TINY, name="big-head", L=3, d_ffn=704, vocab=3000),
+}
+
+
+class Two:
+    """The same weights in a context of either path."""
+
+    def __init__(self, cfg):
+        self.cfg = cfg
+        layers = [{k: v.cuda().contiguous() for k, v in datagen.layer_weights(cfg, l, "cpu").items()} for l in range(cfg.L)]
+        head = {k: v.cuda().contiguous() for k, v in datagen.head_weights(cfg, "cpu").items()}
+        self.eng = []
+        for flags in (0, clasp.FLAG_MULTI_KERNEL):
+            e = clasp.Clasp(clasp.make_config(cfg, max_ctx=200, max_rows=64, max_M=cfg.L, max_T=8, max_head_rows=16, flags=flags))
+            e.load_layers(0, layers)
+            e.load_head(head)
+            self.eng.append(e)
+
+    def caches(self, ctx):
+        out = []
+        for e in self.eng:
+            kv = clasp.KVCache(e.cfg)
+            kv.k[:, :ctx] = datagen.normal_rows(91, 0, tuple(kv.k[:, :ctx].shape)).cuda()
+            kv.v[:, :ctx] = datagen.normal_rows(91, 1, tuple(kv.v[:, :ctx].shape)).cuda()
+            out.append(kv)
+        return out
+
+
+@pytest.fixture(scope="module", params=list(MODELS))
+def two(request):
+    return Two(MODELS[request.param])
+
+
+def close(a, b):
+    return rel_l2(a.double().cpu().numpy(), b.double().cpu().numpy()) < TOL
+
+
+@pytest.mark.parametrize("n,ctx", [(1, 0), (1, 31), (2, 32), (3, 7), (8, 120), (9, 0), (33, 100), (64, 64)])
+def test_forward(two, n, ctx):
+    toks = datagen.token_ids(two.cfg, n).to(torch.int32).cuda()
+    heads = min(n, 9)
+    res = []
+    for e, kv in zip(two.eng, two.caches(ctx)):
+        n0 = e.launch_count()
+        am, hid = e.verify(toks, ctx, kv, heads)
+        res.append((am.cpu(), hid, kv, e.launch_count() - n0))
+        assert e.device_status() == 0
+    (am1, h1, kv1, n1), (am2, h2, kv2, n2) = res
+    assert n1 <= 4 < n2                       # one launch (and three when the head does not fit)
+    assert close(h1, h2) and close(kv1.k, kv2.k) and close(kv1.v, kv2.v)
+    assert torch.equal(am1, am2)
+
+
+@pytest.mark.parametrize("skip", ["none", "some", "all"])
+def test_draft(two, skip):
+    L = two.cfg.L
+    mask = {"none": bytes(L), "some": bytes(l % 2 for l in range(L)), "all": bytes([1] * L)}[skip]
+    res = []
+    for e, kv in zip(two.eng, two.caches(50)):
+        tok = torch.tensor([5], dtype=torch.int32, device="cuda")
+        out, prob = torch.zeros(1, dtype=torch.int32, device="cuda"), torch.zeros(1, device="cuda")
+        e.draft_forward(mask, tok, 50, kv, out, prob)
+        assert e.device_status() == 0
+        res.append((int(out), float(prob), kv))
+    assert res[0][0] == res[1][0] and abs(res[0][1] - res[1][1]) < 1e-5 * res[1][1]
+    assert close(res[0][2].k, res[1][2].k) and close(res[0][2].v, res[1][2].v)
+
+
+@pytest.mark.parametrize("M,T,ctx", [(1, 1, 0), (2, 1, 63), (3, 1, 64), (2, 3, 33), (3, 8, 150)])
+def test_search(two, M, T, ctx):
+    cfg = two.cfg
+    hid = datagen.normal_rows(92, M * 10 + T, (T, cfg.L + 1, cfg.d_model)).to(torch.float32).cuda()
+    res = []
+    for e, kv in zip(two.eng, two.caches(ctx)):
+        res.append(e.dp_search(hid, cfg.d_model, (cfg.L + 1) * cfg.d_model, kv, ctx, ctx, T, M))
+        assert e.device_status() == 0
+    a, b = res
+    # margins of random states are of the order of 1 / sqrt(d): far from ties
+    assert torch.equal(a["S"], b["S"]) and close(a["g_final"], b["g_final"])
+    for key in ("D", "margin"):
+        x, y = a[key], b[key]
+        assert torch.equal(torch.isnan(x), torch.isnan(y))
+        ok = ~torch.isnan(y)
+        assert float((x[ok] - y[ok]).abs().max() if ok.any() else 0.0) < TOL
