@@ -967,6 +967,12 @@ int engine_launch(clasp_ctx* ctx, int Rmax, int head_off, clasp::SetupArgs setup
   const size_t dyn = 1024 + (size_t)ring_pages * pk::PAGE + scratch_bytes;
 
   const int qdim = qd;
+  // A 3-D operand box holds all chunks of a ring item.  Two items that large must fit the largest ring, else no launch
+  // takes the box (and the widest ones are beyond what a tensor map can describe: 8 chunks of 128 or 256 rows).
+  const int ring_most = (optin - ctx->e_static_smem - 1024 - pk::SCRATCH_BYTES) / pk::PAGE;
+  auto box3 = [&](int kind, int row_blocks) {
+    return ctx->e_use3d[kind] && ctx->e_kpi[kind] * row_blocks * b_pages * 2 <= ring_most;
+  };
   auto bm = ctx->e_bmaps.find(BN);
   if (bm == ctx->e_bmaps.end()) {
     std::array<CUtensorMap, 10> m{};
@@ -975,13 +981,13 @@ int engine_launch(clasp_ctx* ctx, int Rmax, int head_off, clasp::SetupArgs setup
     rc |= make_map(ctx, ws.attn, rows_cap, qdim, BN, &m[1]);
     rc |= make_map(ctx, ws.xn_m, rows_cap, d, BN, &m[2]);
     rc |= make_map(ctx, ws.act, rows_cap, c.d_ffn, BN, &m[3]);
-    if (ctx->e_use3d[pk::G_QKV]) rc |= make_map3(ctx, ws.xn, rows_cap, d, BN, ctx->e_kpi[pk::G_QKV], &m[4]);
-    if (ctx->e_use3d[pk::G_O]) rc |= make_map3(ctx, ws.attn, rows_cap, qdim, BN, ctx->e_kpi[pk::G_O], &m[5]);
-    if (ctx->e_use3d[pk::G_GU]) rc |= make_map3(ctx, ws.xn_m, rows_cap, d, BN, ctx->e_kpi[pk::G_GU], &m[6]);
-    if (ctx->e_use3d[pk::G_DOWN]) rc |= make_map3(ctx, ws.act, rows_cap, c.d_ffn, BN, ctx->e_kpi[pk::G_DOWN], &m[7]);
+    if (box3(pk::G_QKV, 1)) rc |= make_map3(ctx, ws.xn, rows_cap, d, BN, ctx->e_kpi[pk::G_QKV], &m[4]);
+    if (box3(pk::G_O, 1)) rc |= make_map3(ctx, ws.attn, rows_cap, qdim, BN, ctx->e_kpi[pk::G_O], &m[5]);
+    if (box3(pk::G_GU, 1)) rc |= make_map3(ctx, ws.xn_m, rows_cap, d, BN, ctx->e_kpi[pk::G_GU], &m[6]);
+    if (box3(pk::G_DOWN, 1)) rc |= make_map3(ctx, ws.act, rows_cap, c.d_ffn, BN, ctx->e_kpi[pk::G_DOWN], &m[7]);
     if (2 * BN <= 256) {
       rc |= make_map(ctx, ws.xn, rows_cap, d, 2 * BN, &m[8]);
-      if (ctx->e_use3d[pk::G_QKV]) rc |= make_map3(ctx, ws.xn, rows_cap, d, 2 * BN, ctx->e_kpi[pk::G_QKV], &m[9]);
+      if (box3(pk::G_QKV, 2)) rc |= make_map3(ctx, ws.xn, rows_cap, d, 2 * BN, ctx->e_kpi[pk::G_QKV], &m[9]);
     }
     if (rc) return CLASP_ERR_CUDA;
     bm = ctx->e_bmaps.emplace(BN, m).first;
@@ -992,7 +998,7 @@ int engine_launch(clasp_ctx* ctx, int Rmax, int head_off, clasp::SetupArgs setup
     std::array<CUtensorMap, 2> m{};
     const bf16* base = (const bf16*)ws.xn + (size_t)head_off * d;
     int rc = make_map(ctx, base, rows_cap - head_off, d, BN, &m[0]);
-    if (ctx->e_use3d[pk::G_HEAD]) rc |= make_map3(ctx, base, rows_cap - head_off, d, BN, ctx->e_kpi[pk::G_HEAD], &m[1]);
+    if (box3(pk::G_HEAD, 1)) rc |= make_map3(ctx, base, rows_cap - head_off, d, BN, ctx->e_kpi[pk::G_HEAD], &m[1]);
     if (rc) return CLASP_ERR_CUDA;
     hm = ctx->e_headmaps.emplace(hk, m).first;
   }

@@ -66,3 +66,16 @@ def test_long_prompt_in_one_call_and_in_pieces(pair):
     assert rel_l2(h1[-last:].cpu().numpy(), h2.cpu().numpy()) < tol_hidden(cfg)
     assert rel_l2(kv1.k[:, :n].float().cpu().numpy(), kv2.k[:, :n].float().cpu().numpy()) < tol_hidden(cfg)
     assert pair.engine.device_status() == 0
+
+
+@pytest.mark.parametrize("n", [112, 113, 128])
+def test_the_widest_calls_of_the_persistent_kernel(pair, n):
+    """128 operand rows: on these narrow models a ring item's operand box would be larger than a tensor map describes."""
+    cfg = pair.cfg
+    toks = torch.randint(0, cfg.vocab, (n,), generator=torch.Generator().manual_seed(9), dtype=torch.int32).cuda()
+    kv1, kv2 = pair.new_kv(), pair.new_kv()
+    _, h1 = pair.engine.verify(toks, 0, kv1, 1)
+    pair.engine.verify(toks[:64], 0, kv2, 0, want_hidden=False)
+    _, h2 = pair.engine.verify(toks[64:], 64, kv2, 1)
+    assert rel_l2(h1[64:].cpu().numpy(), h2.cpu().numpy()) < tol_hidden(cfg)
+    assert pair.engine.device_status() == 0
