@@ -1041,26 +1041,8 @@ int engine_launch(clasp_ctx* ctx, int Rmax, int head_off, clasp::SetupArgs setup
   // position's attention is summed in the same order whichever call computes it (verification and
   // one-token decoding must agree bit for bit).  The search only has to agree with itself: it cuts
   // the keys it sees into at most 32 runs, which spreads a short context over many more CTAs.
-  // Which cut: the (kv head, run or own block, block of 128 pairs) items are dealt out to the CTAs in rounds, and an item
-  // costs its tiles of 32 keys plus ATT_ITEM_TILES tiles' time for its queries and its partial result (step stamps: 1.5 us
-  // per tile, 6 us per item).  One run of 32 keys per CTA is best while that is one round; past it longer runs in fewer
-  // rounds are.
-  if (search_ctx >= 0) {
-    constexpr int ATT_ITEM_TILES = 4;
-    const int n_own = (Rmax + pk::ATT_KEYS - 1) / pk::ATT_KEYS;
-    const int n_pb = (Rmax * (c.n_q_heads / c.n_kv_heads) + 127) / 128;
-    const int keys = std::max(search_ctx, 1);
-    const int len_min = pk::ATT_KEYS * ((keys + pk::ATT_KEYS * 32 - 1) / (pk::ATT_KEYS * 32));   // at most 32 runs
-    int best_len = 0;
-    long best_cost = 0;
-    for (int len = len_min; len < keys + pk::ATT_KEYS; len += pk::ATT_KEYS) {
-      const int runs = (keys + len - 1) / len;
-      const long rounds = ((long)c.n_kv_heads * (runs + n_own) * n_pb + ctx->e_G - 1) / ctx->e_G;
-      const long cost = rounds * (ATT_ITEM_TILES + len / pk::ATT_KEYS);
-      if (best_len == 0 || cost < best_cost) { best_len = len; best_cost = cost; }
-    }
-    P.c.run_len = best_len;
-  }
+  if (search_ctx >= 0) P.c.run_len = pk::ATT_KEYS * ((search_ctx + pk::ATT_KEYS * 32 - 1) / (pk::ATT_KEYS * 32) > 0
+                                                       ? (search_ctx + pk::ATT_KEYS * 32 - 1) / (pk::ATT_KEYS * 32) : 1);
   if (att_tc) {
     // run length: whole 64-key tiles, at most 32 runs; the cut that needs the fewest tile steps when the
     // (kv head, run, pair block) items are dealt out to the CTAs (one more step per round for its set-up)

@@ -6,7 +6,8 @@ at the shape bench.py times.  The oracle's own prefill supplies the objective st
 rounded to the cache dtype, is handed to the device byte for byte.
 
 Tolerances: scores 1e-3, margins 2e-3, decisions identical wherever the oracle's margin exceeds 1e-3
-(cell by cell), hidden states relative L2 <= 2e-2 plus the max-abs guard."""
+(cell by cell), hidden states relative L2 <= 2e-2 plus the max-abs guard.  A last case compares the tables of searches for
+different M, bit for bit."""
 import numpy as np
 import pytest
 import torch
@@ -94,5 +95,28 @@ def test_whole_table_against_oracle(shape, flags):
         np.testing.assert_array_equal(rf["S"].cpu().numpy(), ref["S"])
         assert close_hidden(rf["g_final"].cpu().numpy(), ref["g"][L, M], 2e-2)
         assert eng.device_status() == 0
+    finally:
+        eng.close()
+
+
+def test_table_columns_do_not_depend_on_the_number_of_states(shape):
+    """Column j of the table is the same bits whatever M: a row's attention cuts its keys by the context alone,
+    never by how many rows share the launch.  T = 16, 1024 visible positions: 16 rows against 48."""
+    cfg, C, T = shape.cfg, 1024, 16
+    L, d = cfg.L, cfg.d_model
+    ccfg = shape.clasp.make_config(cfg, max_ctx=C + T, max_rows=64, max_M=3, max_T=T, max_head_rows=4, flags=FLAG_NO_DEFER)
+    eng = shape.clasp.Clasp(ccfg)
+    try:
+        eng.load_layers(0, shape.layers)
+        kv = shape.clasp.KVCache(ccfg)
+        g = torch.Generator(device="cuda").manual_seed(3)
+        kv.k.normal_(generator=g)
+        kv.v.normal_(generator=g)
+        x = torch.randn((T, L + 1, d), device="cuda", generator=g).cumsum(1)      # a random walk over the layers
+        res = [eng.dp_search(x, d, (L + 1) * d, kv, C, C, T, m) for m in (1, 3)]
+        assert eng.device_status() == 0
+        for key in ("D", "margin"):
+            a, b = (r[key][:, :2].nan_to_num(7.0) for r in res)
+            assert torch.equal(a, b)
     finally:
         eng.close()
