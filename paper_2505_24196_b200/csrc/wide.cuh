@@ -209,6 +209,17 @@ struct TileAt {
 };
 
 __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+// Barrier of the eight epilogue warps that also tells whether p holds in any of them.  After a wait each warp polls for itself,
+// and the polls of one may run out just before another's succeed: they go on, or leave, together -- a warp that left alone
+// would be missing at the barriers of the others, which have no limit.
+__device__ __forceinline__ bool epi_any(bool p) {
+  uint32_t r;
+  asm volatile("{\n\t.reg .pred a, b;\n\tsetp.ne.u32 a, %1, 0;\n\tbar.red.or.pred b, 1, 256, a;\n\tselp.u32 %0, 1, 0, b;\n\t}"
+               : "=r"(r)
+               : "r"((uint32_t)p)
+               : "memory");
+  return r != 0;
+}
 
 // y[r, n] = sum_k x[r, k] w[n, k] over tiles of 256 rows x 256 features (SwiGLU: 128 gate and 128 up features).  A pair
 // of CTAs multiplies a tile: each loads 128 rows of x and 128 rows of W, the even CTA issues M = 256 MMAs that read
@@ -324,8 +335,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ C
     while (items.next(p, tile, kb, ke)) {
       const TileAt t(p, tile);
       const uint32_t buf = n_acc & 1u;
-      bool ok = tc::mbar_wait(tc::smem_u32(&acc_full[buf]), (n_acc >> 1) & 1u, p.status, p.spin_fast, p.spin_slow);
-      if (!__all_sync(0xffffffffu, ok)) { s_abort = 1; break; }
+      const bool ok = tc::mbar_wait(tc::smem_u32(&acc_full[buf]), (n_acc >> 1) & 1u, p.status, p.spin_fast, p.spin_slow);
+      __syncwarp();
+      if (epi_any(!ok)) { s_abort = 1; break; }   // (a part of a split tile is then never counted: the status call clears the counters)
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t t_row = tmem_base + buf * TN + ((uint32_t)(quarter * 32) << 16);
       const int r = t.m0 + (int)rank * TM + row_l;

@@ -67,3 +67,26 @@ def test_layer_kernel_wait_that_runs_out_is_reported_and_the_context_recovers(pa
     kv_to_oracle(kv, pair.max_ctx, ocache)
     ref, _, _ = orc.decoder_layer(x[:1].double().numpy(), pair.oracle.layer(2), ocache.k[2], ocache.v[2], 40, 40, cfg)
     assert close_hidden(again[:1].cpu().numpy(), ref, tol_hidden(cfg))
+
+
+@pytest.mark.parametrize("n", [129, 700])
+def test_many_row_kernels_whose_waits_run_out_are_reported_and_the_context_recovers(n):
+    """Layers over more than 128 rows (products with and without split tiles, attention): every launch of the call gives up."""
+    cfg = datagen.CONFIGS["mini8b"]
+    p = Pair(cfg, max_ctx=1024, max_rows=700, max_M=1, max_T=1, max_head_rows=4)
+    eng = p.engine
+    toks = datagen.token_ids(cfg, n).to(torch.int32).cuda()
+    kv = p.new_kv()
+    _, good = eng.verify(toks, 300, kv, 1)
+    assert eng.device_status() == 0
+    for polls in (1, 3, 20):                       # moderate limits: some waits succeed, others run out
+        eng.set_wait_limit(polls)
+        eng.verify(toks, 300, p.new_kv(), 1)
+        status = eng.device_status()
+        assert status == TIMEOUT if polls == 1 else status in (0, TIMEOUT)
+        assert eng.device_status() == 0
+    eng.set_wait_limit(0)
+    _, again = eng.verify(toks, 300, kv, 1)
+    assert eng.device_status() == 0
+    assert torch.equal(again, good)
+    eng.close()
