@@ -26,6 +26,7 @@ constexpr int NR = 8;              // rows per pass of a product
 constexpr int MAX_F = 6;           // features per warp and product
 constexpr int MAX_L = 32;
 constexpr int MAX_STATES = 64;
+constexpr uint32_t GAVE_UP = 1u << 4;
 constexpr int ROW_COS = 128;       // rows of an Eq. 2 step per pass (two doubles each in the attention's area)
 
 struct LayerPtrs {
@@ -124,7 +125,7 @@ struct Call {
   int* s_take;
   uint8_t* s_choice;
   uint64_t* bars;           // per product: its slices of the layer at hand have arrived
-  mutable uint32_t parity;  // bit ph: parity of the next wait on bars[ph]
+  mutable uint32_t parity;  // bit ph: parity of the next wait on bars[ph]; GAVE_UP: a wait of this thread ran out
   int kmax;
   int lo_qkv, n_qkv, lo_d, n_d, lo_f, n_f, lo_v, n_v;
 
@@ -155,7 +156,7 @@ struct Call {
 
   // ---- weight slices of a layer from global to shared memory (one thread; a slice is consecutive rows of a matrix)
   __device__ void fetch(int ph, int l) const {
-    if (tid != 0) return;
+    if (tid != 0 || (parity & GAVE_UP)) return;   // (a barrier whose phase may still be open is not armed again)
     const uint32_t bar = tc::smem_u32(bars + ph);
     auto rows = [&](float* dst, const float* w, int first, int n, int K) {
       if (n > 0) bulk_copy(dst, w + (long long)first * K, (uint32_t)n * K * 4u, bar);
@@ -183,10 +184,15 @@ struct Call {
       rows(w_gu, p.lm_head, lo_v, n_v, p.d);
     }
   }
-  // The slices of product ph have arrived.  A wait that runs out is reported and the call carries on to its end (every
-  // other hand-off is a hardware barrier).
+  // The slices of product ph have arrived.  A wait that runs out is reported and the call carries on to its end through the
+  // hardware barriers of its other hand-offs: the thread polls once per product from then on, and when it is the one that
+  // fetches slices it fetches none (whoever still waits for those runs out in turn, once).
   __device__ __forceinline__ void arrived(int ph) const {
-    if (!tc::mbar_wait(tc::smem_u32(bars + ph), (parity >> ph) & 1u, p.status, p.spin_fast, p.spin_slow)) parity |= 16u;
+    const uint32_t bar = tc::smem_u32(bars + ph), par = (parity >> ph) & 1u;
+    if (!tc::mbar_test(bar, par) && ((parity & GAVE_UP) || !tc::mbar_wait(bar, par, p.status, p.spin_fast, p.spin_slow))) {
+      parity |= GAVE_UP;
+      return;
+    }
     parity ^= 1u << ph;
   }
 
@@ -704,7 +710,7 @@ __global__ void __launch_bounds__(THREADS, 1) call_kernel(const __grid_constant_
   __syncthreads();
   if (p.search) c.search();
   else c.forward();
-  if (c.parity & 16u)   // a wait ran out: copies still in flight land before the shared memory is given back
+  if (c.parity & GAVE_UP)   // a wait ran out: copies still in flight land before the shared memory is given back
     for (int i = 0; i < 2000; ++i) __nanosleep(1000);
 }
 

@@ -3,6 +3,8 @@ forever: the context's wait limit is set to one poll, so the first wait of a hea
 not satisfied at once (a copy still in flight) gives up.  The kernel must then end by itself (copies
 in flight awaited, tensor memory freed), the status call must report CLASP_ERR_TIMEOUT once, and the
 context must work again after the limit is restored."""
+import dataclasses
+
 import pytest
 import torch
 
@@ -89,4 +91,37 @@ def test_many_row_kernels_whose_waits_run_out_are_reported_and_the_context_recov
     _, again = eng.verify(toks, 300, kv, 1)
     assert eng.device_status() == 0
     assert torch.equal(again, good)
+    eng.close()
+
+
+def test_one_cluster_kernel_under_the_shortest_limit_ends_and_the_context_recovers():
+    """The fp32 kernel of a whole call.  Its weight slices are fetched before the first rows are ready and then a layer
+    ahead, so that even a limit of one poll is hardly ever reached on a healthy launch: the status may be either, the call
+    ends and the context computes the same bits afterwards.  (That the call winds down when a wait does run out is shown
+    by reading: the thread that gave up arms no barrier again, the other hand-offs are barriers that all threads reach.)"""
+    cfg = dataclasses.replace(datagen.CONFIGS["tiny"], name="large-slices", L=4, d_model=384, n_q_heads=8, n_kv_heads=8, d_ffn=16)
+    p = Pair(cfg, max_ctx=64, max_rows=16, max_M=2, max_T=1, max_head_rows=4)
+    eng = p.engine
+    toks = datagen.token_ids(cfg, 3).to(torch.int32).cuda()
+    kv = p.new_kv()
+    n0 = eng.launch_count()
+    _, good = eng.verify(toks, 20, kv, 0)
+    assert eng.launch_count() - n0 == 1
+    s_good = eng.dp_search(good[2], cfg.d_model, 0, kv, 22, 22, 1, 2)
+    assert eng.device_status() == 0
+    flush = torch.empty(256 << 20, dtype=torch.uint8, device="cuda")
+    eng.set_wait_limit(1)
+    for _ in range(4):
+        flush.zero_()                               # (the weights come from memory, not from L2)
+        eng.verify(toks, 20, p.new_kv(), 0)
+        assert eng.device_status() in (0, TIMEOUT)
+        eng.dp_search(good[2], cfg.d_model, 0, kv, 22, 22, 1, 2)
+        assert eng.device_status() in (0, TIMEOUT)
+        assert eng.device_status() == 0
+    eng.set_wait_limit(0)
+    _, again = eng.verify(toks, 20, kv, 0)
+    s_again = eng.dp_search(good[2], cfg.d_model, 0, kv, 22, 22, 1, 2)
+    assert eng.device_status() == 0
+    assert torch.equal(again, good) and torch.equal(s_again["S"], s_good["S"])
+    assert torch.equal(s_again["g_final"], s_good["g_final"])
     eng.close()
