@@ -242,6 +242,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
     bool ok = true;
     if (have_acc) ok = mbar_wait(smem_u32(&bar_accum), 0, p.status, p.spin_fast, p.spin_slow);
     ok = __all_sync(0xffffffffu, ok);  // tcgen05.ld below needs the whole warp
+    if (!ok) s_abort = 1;              // (multiplies may still be in flight although the other warps' waits succeeded)
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t t_lane = tmem_base + ((uint32_t)(q * 32) << 16);
     const int planes = p.dual ? 2 : 1;
