@@ -206,6 +206,7 @@ struct Call {
         // (rows of up to 256 columns stay in registers, their norm weights come in the same trip)
         float4 v[2], g[2];
         float ss = 0.f;
+        double tail = 0.0;   // (past 256 columns: a lane's sum of many groups of four loses what a small group adds)
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
           const int c = lane * 4 + q * 128;
@@ -219,9 +220,10 @@ struct Call {
         for (int q = 0; q < 2; ++q) ss += v[q].x * v[q].x + v[q].y * v[q].y + v[q].z * v[q].z + v[q].w * v[q].w;
         for (int c = lane * 4 + 256; c < K; c += 128) {
           const float4 u = __ldcg(reinterpret_cast<const float4*>(x + c));
-          ss += u.x * u.x + u.y * u.y + u.z * u.z + u.w * u.w;
+          tail += (double)(u.x * u.x + u.y * u.y + u.z * u.z + u.w * u.w);
           *reinterpret_cast<float4*>(dst + c) = u;
         }
+        if (K > 256) ss = (float)((double)ss + tail);
         const float sc = rsqrtf(warp_sum(ss) / (float)K + p.eps);
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
@@ -589,20 +591,19 @@ struct Call {
         const float* x = p.hidden + (long long)i * p.layer_stride + t * p.token_stride;
         const float* s = skip_row(g_prev, i, r);
         const float* y = j <= n ? p.G + (long long)r * p.d : s;
-        float v[5] = {0.f, 0.f, 0.f, 0.f, 0.f};   // x.x, y.y, x.y, s.s, x.s
+        double q[5] = {0.0, 0.0, 0.0, 0.0, 0.0};   // x.x, y.y, x.y, s.s, x.s: four products in fp32, the rest in double
 #pragma unroll 2
         for (int c = lane * 4; c < p.d; c += 128) {
           const float4 a = __ldg(reinterpret_cast<const float4*>(x + c));
           const float4 b = __ldcg(reinterpret_cast<const float4*>(y + c)), e = __ldcg(reinterpret_cast<const float4*>(s + c));
-          v[0] += a.x * a.x + a.y * a.y + a.z * a.z + a.w * a.w;
-          v[1] += b.x * b.x + b.y * b.y + b.z * b.z + b.w * b.w;
-          v[2] += a.x * b.x + a.y * b.y + a.z * b.z + a.w * b.w;
-          v[3] += e.x * e.x + e.y * e.y + e.z * e.z + e.w * e.w;
-          v[4] += a.x * e.x + a.y * e.y + a.z * e.z + a.w * e.w;
+          q[0] += (double)(a.x * a.x + a.y * a.y + a.z * a.z + a.w * a.w);
+          q[1] += (double)(b.x * b.x + b.y * b.y + b.z * b.z + b.w * b.w);
+          q[2] += (double)(a.x * b.x + a.y * b.y + a.z * b.z + a.w * b.w);
+          q[3] += (double)(e.x * e.x + e.y * e.y + e.z * e.z + e.w * e.w);
+          q[4] += (double)(a.x * e.x + a.y * e.y + a.z * e.z + a.w * e.w);
         }
-        double q[5];
 #pragma unroll
-        for (int k = 0; k < 5; ++k) q[k] = warp_sum_d((double)v[k]);
+        for (int k = 0; k < 5; ++k) q[k] = warp_sum_d(q[k]);
         if (lane == 0) {
           const double nx = fmax(sqrt(q[0]), 1e-12);
           row_cos[r - r0] = make_double2(q[2] / (nx * fmax(sqrt(q[1]), 1e-12)), q[4] / (nx * fmax(sqrt(q[3]), 1e-12)));

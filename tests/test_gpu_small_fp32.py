@@ -105,3 +105,49 @@ def test_search(two, M, T, ctx):
         assert torch.equal(torch.isnan(x), torch.isnan(y))
         ok = ~torch.isnan(y)
         assert float((x[ok] - y[ok]).abs().max() if ok.any() else 0.0) < TOL
+
+
+def test_cosines_keep_small_columns():
+    """Eq. 2's sums over many columns: 128 columns of 1 and 1408 of about 2^-12.5, of the other sign in one state.  An
+    addend of four small products is below half an ulp of a lane's fp32 sum, all of them together move the cosine by
+    6.4e-7; partial sums of at most four products leave 2^-24 or so."""
+    cfg = dataclasses.replace(TINY, name="wide-row", L=2, d_model=1536, n_q_heads=1, n_kv_heads=1, head_dim=64, d_ffn=32, vocab=64)
+    e = clasp.Clasp(clasp.make_config(cfg, max_ctx=8, max_rows=4, max_M=2, max_T=1))
+    e.load_layers(0, [{k: v.cuda().contiguous() for k, v in datagen.layer_weights(cfg, l, "cpu").items()} for l in range(cfg.L)])
+    small = torch.tensor(1.7e-4)
+    x0 = torch.ones(1536)
+    x0[128:] = small
+    x1 = x0.clone()
+    x1[128:] = -small
+    hid = torch.stack([x0, x1, x0]).cuda()
+    n0 = e.launch_count()
+    r = e.dp_search(hid, 1536, 0, clasp.KVCache(e.cfg), 0, 0, 1, 2)
+    assert e.launch_count() - n0 == 1 and e.device_status() == 0
+    a, b = x1.double(), x0.double()
+    want = float(a @ b / (a.norm() * b.norm()))
+    assert abs(float(r["D"][1, 1]) - want) < 2.0 ** -22
+    e.close()
+
+
+def test_norm_keeps_small_columns():
+    """The same for the sum of squares of an RMSNorm: 128 columns of 1 and 1408 of 2^-12.5 are 6.2e-7 of the sum, half that
+    of the scale.  wv of one column copies the normed column 0 into the value cache."""
+    cfg = dataclasses.replace(TINY, name="wide-row", L=1, d_model=1536, n_q_heads=1, n_kv_heads=1, head_dim=64, d_ffn=32, vocab=64)
+    lw = {k: v.cuda().contiguous() for k, v in datagen.layer_weights(cfg, 0, "cpu").items()}
+    head = {k: v.cuda().contiguous() for k, v in datagen.head_weights(cfg, "cpu").items()}
+    lw["attn_norm"].fill_(1.0)
+    lw["wv"].zero_()
+    lw["wv"][:, 0] = 1.0
+    head["embed"][:, :128] = 1.0
+    head["embed"][:, 128:] = 1.7e-4
+    e = clasp.Clasp(clasp.make_config(cfg, max_ctx=8, max_rows=4, max_M=1, max_T=1))
+    e.load_layers(0, [lw])
+    e.load_head(head)
+    kv = clasp.KVCache(e.cfg)
+    n0 = e.launch_count()
+    e.verify(torch.zeros(1, dtype=torch.int32, device="cuda"), 0, kv, 0)
+    assert e.launch_count() - n0 == 1 and e.device_status() == 0
+    row = head["embed"][0].double()
+    want = float(torch.rsqrt((row * row).mean() + cfg.rms_eps))
+    assert abs(float(kv.v[0, 0, 0, 0]) / want - 1.0) < 2.0 ** -23
+    e.close()
