@@ -664,7 +664,7 @@ int s32_launch_config(clasp_ctx* ctx, cudaLaunchConfig_t* lc, cudaLaunchAttribut
 int s32_setup(clasp_ctx* ctx) {
   const clasp_config& c = ctx->cfg;
   ctx->use_s32 = ctx->s32_head = false;
-  if (c.dtype != CLASP_FP32 || (c.flags & (CLASP_FLAG_MULTI_KERNEL | CLASP_FLAG_PRUNE))) return CLASP_OK;
+  if (c.dtype != CLASP_FP32 || (c.flags & CLASP_FLAG_MULTI_KERNEL)) return CLASP_OK;
   const int d = c.d_model, qd = c.n_q_heads * c.head_dim, kvd = c.n_kv_heads * c.head_dim, cap = s32::MAX_F * s32::WARPS;
   if (c.L > s32::MAX_L || c.max_M + 1 > s32::MAX_STATES || s32::slice_cap(qd + 2 * kvd) > cap || s32::slice_cap(d) > cap ||
       2 * s32::slice_cap(c.d_ffn) > cap)
@@ -1326,6 +1326,7 @@ int clasp_dp_search(clasp_ctx* ctx, const float* hidden_states, int64_t layer_st
     s32_params(ctx, &p, T, ctx_len, pos0);
     for (int l = 0; l < L; ++l) s32_layer(ctx, &p, l, kv[l]);
     p.search = 1; p.hidden = hidden_states; p.layer_stride = layer_stride; p.token_stride = token_stride; p.M = M;
+    p.prune = (c.flags & CLASP_FLAG_PRUNE) != 0;
     p.G = ws.G; p.g[0] = ws.grow[0]; p.g[1] = ws.grow[1];
     p.scores = scores; p.margins = margins; p.g_final = g_final; p.forced = forced_choice; p.skip_mask = skip_mask;
     return s32_launch(ctx, &p);

@@ -56,8 +56,8 @@ struct Params {
   // search
   const float* hidden;
   long long layer_stride, token_stride;
-  int M;
-  float* G;
+  int M, prune;             // prune: only states that can reach (L, M)
+  float* G;                 // layer output of state j, row t at row (j - 1) * T + t
   float* g[2];
   float *scores, *margins, *g_final;
   const uint8_t* forced;
@@ -575,16 +575,17 @@ struct Call {
     }
   }
 
-  // ---- Eq. 2 step i over n candidate states (plus the diagonal one): every CTA computes all sums and decides alike.
-  // Layer outputs in G, skip candidates in g_prev (state 1's: the objective rows of step i - 1).
+  // ---- Eq. 2 step i over the candidate states j_lo..n (plus the diagonal one): every CTA computes all sums and decides alike.
+  // Layer outputs in G, skip candidates in g_prev (state 1's: the objective rows of step i - 1).  Rows are counted from state
+  // 1's on, whatever j_lo.
   __device__ __forceinline__ const float* skip_row(const float* g_prev, int i, int r) const {
     return r < p.T ? p.hidden + (long long)(i - 1) * p.layer_stride + r * p.token_stride : g_prev + (long long)r * p.d;
   }
-  __device__ void select(int i, int n, bool diag, const float* g_prev, float* g_next) const {
+  __device__ void select(int i, int j_lo, int n, bool diag, const float* g_prev, float* g_next) const {
     const int states = n + (diag ? 1 : 0);
     const int per_pass = max(1, ROW_COS / p.T) * p.T;   // whole states
     double2* row_cos = reinterpret_cast<double2*>(att_q);   // per row (cosine of the layer output, of the skip candidate)
-    for (int r0 = 0; r0 < states * p.T; r0 += per_pass) {
+    for (int r0 = (j_lo - 1) * p.T; r0 < states * p.T; r0 += per_pass) {
       const int r1 = min(states * p.T, r0 + per_pass);
       for (int r = r0 + warp; r < r1; r += WARPS) {
         const int j = r / p.T + 1, t = r % p.T;
@@ -638,7 +639,7 @@ struct Call {
       if (rank == 0) p.scores[(long long)i * (p.M + 1)] = 1.0f;
     }
     __syncthreads();
-    for (int r = rank + warp * CTAS; r < states * p.T; r += CTAS * WARPS) {
+    for (int r = (j_lo - 1) * p.T + rank + warp * CTAS; r < states * p.T; r += CTAS * WARPS) {
       const int j = r / p.T + 1, t = r % p.T;
       const float* src = s_take[j - 1] ? p.G + (long long)r * p.d : skip_row(g_prev, i, r);
       for (int c = lane * 4; c < p.d; c += 128) {
@@ -661,19 +662,27 @@ struct Call {
     }
     for (int c = tid; c < (L + 1) * (M + 1); c += THREADS) s_choice[c] = c == 0 ? 0 : 255;
     __syncthreads();
-    // layer 0 is never applied (its only input would be x_0, whose image is x_1): its slices were not fetched
+    // Layer 0 is never applied (its only input would be x_0, whose image is x_1): its slices were not fetched.  Nor are any
+    // when pruning leaves the diagonal only (M = L).  Pruned steps carry states j_lo..n: from j < M - (L - i) there is no way
+    // to (L, M).  Rows and their sums are the same as without.
     const float* g_prev = p.g[0];
     float* g_next = p.g[1];
     for (int i = 1; i <= L; ++i) {
-      const int n = min(i - 1, M);
-      if (n > 0) {
+      const int n = min(i - 1, M), j_lo = p.prune ? max(1, M - (L - i)) : 1;
+      const int sh = (j_lo - 1) * p.T;   // rows before state j_lo
+      if (n >= j_lo) {
         // the rows the last step chose, straight from where they are (g[i-1] itself is on its way to memory)
         const float* gp = g_next;      // g[i - 2] (ping-pong: the buffer this step overwrites)
-        auto in = [&](int r) -> const float* { return s_take[r / p.T] ? p.G + (long long)r * p.d : skip_row(gp, i - 1, r); };
-        auto res = [&](int r) -> const float* { return g_prev + (long long)(r + p.T) * p.d; };
-        layer(i - 1, n * p.T, false, in, res, [&](int r) { return p.G + (long long)r * p.d; });
+        auto in = [&](int k) -> const float* {
+          const int r = sh + k;
+          return s_take[r / p.T] ? p.G + (long long)r * p.d : skip_row(gp, i - 1, r);
+        };
+        auto res = [&](int k) -> const float* { return g_prev + (long long)(sh + k + p.T) * p.d; };
+        layer(i - 1, n * p.T - sh, false, in, res, [&](int k) { return p.G + (long long)(sh + k) * p.d; });
+      } else if (i > 1) {
+        cluster_barrier();   // the rows the last step wrote
       }
-      select(i, n, i <= M, g_prev, g_next);
+      select(i, j_lo, n, i <= M, g_prev, g_next);
       const float* t = g_prev;
       g_prev = g_next;
       g_next = const_cast<float*>(t);
@@ -706,7 +715,7 @@ __global__ void __launch_bounds__(THREADS, 1) call_kernel(const __grid_constant_
     for (int ph = 0; ph < 4; ++ph) tc::mbar_init(tc::smem_u32(bars + ph), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    for (int ph = 0; ph < 4; ++ph) c.fetch(ph, p.search ? 1 : 0);
+    for (int ph = 0; ph < 4; ++ph) c.fetch(ph, !p.search ? 0 : (p.prune && p.M == p.n_layers ? p.n_layers : 1));
   }
   __syncthreads();
   if (p.search) c.search();

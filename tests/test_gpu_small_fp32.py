@@ -32,6 +32,7 @@ class Two:
         self.cfg = cfg
         layers = [{k: v.cuda().contiguous() for k, v in datagen.layer_weights(cfg, l, "cpu").items()} for l in range(cfg.L)]
         head = {k: v.cuda().contiguous() for k, v in datagen.head_weights(cfg, "cpu").items()}
+        self.layers, self.head = layers, head
         self.eng = []
         for flags in (0, clasp.FLAG_MULTI_KERNEL):
             e = clasp.Clasp(clasp.make_config(cfg, max_ctx=200, max_rows=64, max_M=cfg.L, max_T=8, max_head_rows=16, flags=flags))
@@ -105,6 +106,37 @@ def test_search(two, M, T, ctx):
         assert torch.equal(torch.isnan(x), torch.isnan(y))
         ok = ~torch.isnan(y)
         assert float((x[ok] - y[ok]).abs().max() if ok.any() else 0.0) < TOL
+
+
+@pytest.mark.parametrize("M,T,ctx", [(1, 1, 40), (2, 3, 64), (3, 2, 33), (3, 8, 150)])
+def test_pruned_search_is_the_same_bits(two, M, T, ctx):
+    """CLASP_FLAG_PRUNE: skip set, g[L][M] and every cell that can reach (L, M) unchanged, the others NaN; M = L too
+    (no state is ever pushed through a layer).  A context with the flag keeps the one-launch path for everything."""
+    cfg = two.cfg
+    L = cfg.L
+    hid = datagen.normal_rows(93, M * 10 + T, (T, L + 1, cfg.d_model)).to(torch.float32).cuda()
+    e, kv = two.eng[0], two.caches(ctx)[0]
+    p = clasp.Clasp(clasp.make_config(cfg, max_ctx=200, max_rows=64, max_M=L, max_T=8, max_head_rows=16, flags=clasp.FLAG_PRUNE))
+    p.load_layers(0, two.layers)
+    p.load_head(two.head)
+    try:
+        for m in (M, L):
+            n0 = p.launch_count()
+            a, b = (x.dp_search(hid, cfg.d_model, (L + 1) * cfg.d_model, kv, ctx, ctx, T, m) for x in (e, p))
+            assert p.launch_count() - n0 == 1
+            assert p.device_status() == 0 and e.device_status() == 0
+            i, j = torch.meshgrid(torch.arange(L + 1, device="cuda"), torch.arange(m + 1, device="cuda"), indexing="ij")
+            out = (j < m - (L - i)) & (j > 0)
+            assert torch.equal(a["S"], b["S"]) and torch.equal(a["g_final"], b["g_final"])
+            for key in ("D", "margin"):
+                want = a[key].masked_fill(out, float("nan"))
+                assert torch.equal(torch.isnan(b[key]), torch.isnan(want)), (m, key)
+                assert torch.equal(b[key].nan_to_num(7.0), want.nan_to_num(7.0)), (m, key)
+        n0 = p.launch_count()
+        p.verify(torch.zeros(4, dtype=torch.int32, device="cuda"), ctx, kv, 1)
+        assert p.launch_count() - n0 <= 4
+    finally:
+        p.close()
 
 
 def test_cosines_keep_small_columns():
