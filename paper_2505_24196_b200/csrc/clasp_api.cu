@@ -283,6 +283,30 @@ struct GemmCall {
   bool wide = false;         // a decoder layer's product over many rows (gemm_wide)
 };
 
+// Launch timing (clasp_profile_gemm): a pair of events around a launch, and the weight bytes it has to read.
+int profile_begin(clasp_ctx* ctx) {
+  if (!ctx->profiling) return CLASP_OK;
+  cudaEvent_t e0, e1;
+  if (cudaEventCreate(&e0) != cudaSuccess) return CLASP_ERR_CUDA;
+  if (cudaEventCreate(&e1) != cudaSuccess) {
+    cudaEventDestroy(e0);
+    return CLASP_ERR_CUDA;
+  }
+  cudaEventRecord(e0, ctx->stream);
+  ctx->prof_events.emplace_back(e0, e1);
+  return CLASP_OK;
+}
+void profile_end(clasp_ctx* ctx, double bytes) {
+  if (!ctx->profiling) return;
+  cudaEventRecord(ctx->prof_events.back().second, ctx->stream);
+  ctx->prof_bytes += bytes;
+}
+double weight_bytes(const GemmCall& g) {
+  double nk = 0.0;
+  for (int m = 0; m < g.n_mats; ++m) nk += (double)g.N[m] * g.K;
+  return nk * 2.0 * (g.epi == clasp::EPI_SWIGLU ? 2 : 1);
+}
+
 template <typename TW, int EPI>
 int gemm_simt_one(clasp_ctx* ctx, const GemmCall& g, int m) {
   constexpr int WARPS = 8, RB = 4;
@@ -369,21 +393,11 @@ int gemm_tc(clasp_ctx* ctx, const GemmCall& g) {
     const CUtensorMap* a1 = dual ? g.w2map : (g.n_mats > 1 ? g.wmap[1] : g.wmap[0]);
     const CUtensorMap* a2 = g.n_mats > 2 ? g.wmap[2] : g.wmap[0];
     dim3 grid(tiles_total, p.splits), block(THREADS);
-    cudaEvent_t e0 = nullptr, e1 = nullptr;
-    if (ctx->profiling) {
-      if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) return CLASP_ERR_CUDA;
-      cudaEventRecord(e0, ctx->stream);
-    }
-    gemm_tc_kernel<<<grid, block, smem, ctx->stream>>>(*a0, *a1, *a2, it->second, p);
-    if (ctx->profiling) {
-      cudaEventRecord(e1, ctx->stream);
-      ctx->prof_events.emplace_back(e0, e1);
-      double nk = 0.0;
-      for (int m = 0; m < g.n_mats; ++m) nk += (double)g.N[m] * g.K;
-      ctx->prof_bytes += nk * 2.0 * (dual + 1);
-    }
-    int rc = launch_check(ctx);
+    int rc = profile_begin(ctx);
     if (rc) return rc;
+    gemm_tc_kernel<<<grid, block, smem, ctx->stream>>>(*a0, *a1, *a2, it->second, p);
+    profile_end(ctx, weight_bytes(g));
+    if ((rc = launch_check(ctx))) return rc;
   }
   return CLASP_OK;
 }
@@ -439,7 +453,9 @@ int gemm_wide(clasp_ctx* ctx, const GemmCall& g) {
   const CUtensorMap* w0 = g.wmap[0];
   const CUtensorMap* w1 = p.dual ? g.w2map : (g.n_mats > 1 ? g.wmap[1] : w0);
   const CUtensorMap* w2 = g.n_mats > 2 ? g.wmap[2] : w0;
+  if ((rc = profile_begin(ctx))) return rc;
   wd::gemm_kernel<<<2 * W, wd::GEMM_THREADS, wd::GEMM_SMEM, ctx->stream>>>(*mx, *w0, *w1, *w2, p);
+  profile_end(ctx, weight_bytes(g));
   return launch_check(ctx);
 }
 
@@ -1078,10 +1094,9 @@ int engine_launch(clasp_ctx* ctx, int Rmax, int head_off, clasp::SetupArgs setup
   P.wait_fast = ctx->wait_limit ? (ctx->wait_limit < pk::WAIT_FAST ? ctx->wait_limit : pk::WAIT_FAST) : pk::WAIT_FAST;
   P.wait_slow = ctx->wait_limit ? ctx->wait_limit : pk::WAIT_SLOW;
 
-  cudaEvent_t e0 = nullptr, e1 = nullptr;
-  if (ctx->profiling) {
-    if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) return CLASP_ERR_CUDA;
-    cudaEventRecord(e0, ctx->stream);
+  {
+    const int rc = profile_begin(ctx);
+    if (rc) return rc;
   }
   void* args[] = {(void*)&bm->second[0], (void*)&bm->second[1], (void*)&bm->second[2], (void*)&bm->second[3],
                   (void*)&hm->second[0], (void*)&bm->second[4], (void*)&bm->second[5], (void*)&bm->second[6],
@@ -1090,9 +1105,9 @@ int engine_launch(clasp_ctx* ctx, int Rmax, int head_off, clasp::SetupArgs setup
   cudaError_t err = cudaLaunchCooperativeKernel(kern, dim3(ctx->e_G), dim3(pk::THREADS),
                                                 args, dyn, ctx->stream);
   if (ctx->profiling) {
-    cudaEventRecord(e1, ctx->stream);
-    ctx->prof_events.emplace_back(e0, e1);
-    for (const pk::Job& J : ctx->e_jobs) ctx->prof_bytes += job_bytes(ctx, J);
+    double bytes = 0.0;
+    for (const pk::Job& J : ctx->e_jobs) bytes += job_bytes(ctx, J);
+    profile_end(ctx, bytes);
   }
   ctx->launches += 1;
   return err == cudaSuccess ? CLASP_OK : CLASP_ERR_CUDA;

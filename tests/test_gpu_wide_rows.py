@@ -1,6 +1,8 @@
 """One decoder layer over more rows than the skinny products take (the tensor-core products and attention of
 csrc/wide.cuh) against the oracle: edges of the 256-row and 256-feature tiles, ragged key tiles, several states with
 their own rows only, key splits, and a row maximum that moves in mid-cache (the rescaling path)."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -79,3 +81,15 @@ def test_the_widest_calls_of_the_persistent_kernel(pair, n):
     _, h2 = pair.engine.verify(toks[64:], 64, kv2, 1)
     assert rel_l2(h1[64:].cpu().numpy(), h2.cpu().numpy()) < tol_hidden(cfg)
     assert pair.engine.device_status() == 0
+
+
+def test_products_are_in_the_launch_timing(pair):
+    """clasp_profile_gemm counts every tensor-core product: four per layer over many rows and the head."""
+    cfg, eng = pair.cfg, pair.engine
+    n, ms, nb = ctypes.c_int64(), ctypes.c_double(), ctypes.c_double()
+    toks = torch.zeros(300, dtype=torch.int32, device="cuda")
+    assert eng.lib.clasp_profile_gemm(eng.handle, 1, None, None, None) == 0
+    eng.verify(toks, 0, pair.new_kv(), 1, want_hidden=False)
+    assert eng.lib.clasp_profile_gemm(eng.handle, 0, ctypes.byref(n), ctypes.byref(ms), ctypes.byref(nb)) == 0
+    assert n.value == 4 * cfg.L + 1 and ms.value > 0.0
+    assert nb.value == cfg.L * cfg.layer_matrix_bytes() + cfg.vocab * cfg.d_model * 2
