@@ -59,15 +59,19 @@ __device__ __forceinline__ uint32_t elect_one() {
   asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(pred));
   return pred;
 }
-// The pair's even CTA: clearing this bit of a shared-memory address names the same place there.
-constexpr uint32_t LEADER_MASK = 0xFEFFFFFFu;
-// a load into this CTA's shared memory that reports its bytes to the even CTA's barrier
+// the same place in the shared memory of the pair's even CTA
+__device__ __forceinline__ uint32_t leader_addr(uint32_t a) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(a));
+  return r;
+}
+// a load into this CTA's shared memory that reports its bytes to a barrier of the even CTA (leader_addr)
 __device__ __forceinline__ void tma_load_pair(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y, uint64_t policy) {
   asm volatile(
       "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
       " [%0], [%1, {%3, %4}], [%2], %5;"
       :
-      : "r"(dst), "l"(map), "r"(bar & LEADER_MASK), "r"(x), "r"(y), "l"(policy)
+      : "r"(dst), "l"(map), "r"(bar), "r"(x), "r"(y), "l"(policy)
       : "memory");
 }
 __device__ __forceinline__ void mma_pair(uint32_t d, uint64_t da, uint64_t db, uint32_t idesc, bool acc, uint32_t el) {
@@ -89,11 +93,7 @@ __device__ __forceinline__ void commit_pair(uint32_t bar, uint32_t el) {
       : "memory");
 }
 __device__ __forceinline__ void arrive_leader(uint32_t bar) {
-  asm volatile(
-      "{\n\t.reg .b32 a;\n\t"
-      "mapa.shared::cluster.u32 a, %0, 0;\n\t"
-      "mbarrier.arrive.release.cluster.shared::cluster.b64 _, [a];\n\t}" ::"r"(bar)
-      : "memory");
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(leader_addr(bar)) : "memory");
 }
 // eight floats (32 bytes): one access where the address allows it.  Predicated inside the statement: the warp stays
 // converged for the tensor-memory reads around it.
@@ -284,10 +284,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ C
           const uint32_t s = n % STAGES;
           if (!tc::mbar_wait(tc::smem_u32(&bar_empty[s]), ((n / STAGES) & 1u) ^ 1u, p.status, p.spin_fast, p.spin_slow)) { ok = false; break; }
           const uint32_t full = tc::smem_u32(&bar_full[s]);
-          const uint32_t dst = ring + s * STAGE_BYTES;
+          const uint32_t dst = ring + s * STAGE_BYTES, full0 = leader_addr(full);
           if (rank == 0) tc::mbar_expect_tx(full, 2 * STAGE_BYTES);
-          tma_load_pair(dst, &map_x, full, k * BK, xy, pol);
-          tma_load_pair(dst + TM * BK * 2, mw, full, k * BK, wy, pol);
+          tma_load_pair(dst, &map_x, full0, k * BK, xy, pol);
+          tma_load_pair(dst + TM * BK * 2, mw, full0, k * BK, wy, pol);
         }
       }
       if (!ok) s_abort = 1;
