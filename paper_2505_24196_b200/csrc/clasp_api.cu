@@ -32,7 +32,7 @@ using bf16 = __nv_bfloat16;
 // 404, 233 / 413, 555 / 462; 16 rows at 500 506 / 709; 32 rows at 1000 1368 / 1095; 64 rows at 0 / 500 946 / 1708, 1957 /
 // 1707; 128 rows at 0 / 500 2360 / 2957, 4037 / 2965; searches of 16 rows at 1000 524 / 650, 32 rows at 500 / 1500
 // 704 / 943, 1248 / 1028.
-constexpr int S32_MAX_ROWS = 128, S32_MAX_KEYS = 2048;
+constexpr int S32_MAX_KEYS = 2048;
 constexpr long long S32_MAX_SCORES = 65536;   // rows x query heads x keys
 constexpr int WIDE_MIN_ROWS = 128;   // layers over more rows take the products and the attention of wide.cuh
 constexpr int MAX_COUNTERS = 4096;   // tiles of one GEMM launch that may use split-K
@@ -745,7 +745,7 @@ void s32_layer(clasp_ctx* ctx, s32::Params* p, int l, const clasp_kv_layer& kv) 
 }
 
 bool s32_takes(const clasp_ctx* ctx, int rows, int keys) {
-  return ctx->use_s32 && rows <= S32_MAX_ROWS && keys <= S32_MAX_KEYS &&
+  return ctx->use_s32 && rows <= s32::MAX_ROWS && keys <= S32_MAX_KEYS &&
          (long long)rows * ctx->cfg.n_q_heads * keys <= S32_MAX_SCORES;
 }
 
@@ -1336,7 +1336,7 @@ int clasp_dp_search(clasp_ctx* ctx, const float* hidden_states, int64_t layer_st
     return CLASP_ERR_INVALID_ARG;
   if (M > 0 && !layers_ready(ctx)) return CLASP_ERR_NOT_LOADED;
   Workspace& ws = ctx->ws;
-  if (M > 0 && T <= s32::ROW_COS && s32_takes(ctx, M * T, ctx_len + T)) {
+  if (M > 0 && s32_takes(ctx, M * T, ctx_len + T)) {
     s32::Params p;
     s32_params(ctx, &p, T, ctx_len, pos0);
     for (int l = 0; l < L; ++l) s32_layer(ctx, &p, l, kv[l]);

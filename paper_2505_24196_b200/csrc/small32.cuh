@@ -27,7 +27,7 @@ constexpr int MAX_F = 6;           // features per warp and product
 constexpr int MAX_L = 32;
 constexpr int MAX_STATES = 64;
 constexpr uint32_t GAVE_UP = 1u << 4;
-constexpr int ROW_COS = 128;       // rows of an Eq. 2 step per pass (two doubles each in the attention's area)
+constexpr int MAX_ROWS = 128;      // rows of a call: an Eq. 2 step keeps two doubles of each in the attention's area
 
 struct LayerPtrs {
   const float *attn_norm, *wq, *wk, *wv, *wo, *mlp_norm, *wg, *wu, *wd;
@@ -66,6 +66,7 @@ struct Params {
   uint32_t spin_fast, spin_slow;
 };
 static_assert(sizeof(Params) < 4000, "kernel parameters");
+static_assert(MAX_ROWS * 2 * (int)sizeof(double) <= WARPS * (2 * 64 + 4) * (int)sizeof(float), "cosines of a step's rows");
 
 __host__ __device__ __forceinline__ int slice_cap(int n) { return (n + CTAS - 1) / CTAS; }
 // floats of dynamic shared memory: weight slices (the gate/up area also takes the head's slice), rows, attention, tables
@@ -582,64 +583,60 @@ struct Call {
     return r < p.T ? p.hidden + (long long)(i - 1) * p.layer_stride + r * p.token_stride : g_prev + (long long)r * p.d;
   }
   __device__ void select(int i, int j_lo, int n, bool diag, const float* g_prev, float* g_next) const {
-    const int states = n + (diag ? 1 : 0);
-    const int per_pass = max(1, ROW_COS / p.T) * p.T;   // whole states
+    const int states = n + (diag ? 1 : 0), r0 = (j_lo - 1) * p.T, r1 = states * p.T;
     double2* row_cos = reinterpret_cast<double2*>(att_q);   // per row (cosine of the layer output, of the skip candidate)
-    for (int r0 = (j_lo - 1) * p.T; r0 < states * p.T; r0 += per_pass) {
-      const int r1 = min(states * p.T, r0 + per_pass);
-      for (int r = r0 + warp; r < r1; r += WARPS) {
-        const int j = r / p.T + 1, t = r % p.T;
-        const float* x = p.hidden + (long long)i * p.layer_stride + t * p.token_stride;
-        const float* s = skip_row(g_prev, i, r);
-        const float* y = j <= n ? p.G + (long long)r * p.d : s;
-        double q[5] = {0.0, 0.0, 0.0, 0.0, 0.0};   // x.x, y.y, x.y, s.s, x.s: four products in fp32, the rest in double
+    for (int r = r0 + warp; r < r1; r += WARPS) {
+      const int j = r / p.T + 1, t = r % p.T;
+      const float* x = p.hidden + (long long)i * p.layer_stride + t * p.token_stride;
+      const float* s = skip_row(g_prev, i, r);
+      const float* y = j <= n ? p.G + (long long)r * p.d : s;
+      double q[5] = {0.0, 0.0, 0.0, 0.0, 0.0};   // x.x, y.y, x.y, s.s, x.s: four products in fp32, the rest in double
 #pragma unroll 2
-        for (int c = lane * 4; c < p.d; c += 128) {
-          const float4 a = __ldg(reinterpret_cast<const float4*>(x + c));
-          const float4 b = __ldcg(reinterpret_cast<const float4*>(y + c)), e = __ldcg(reinterpret_cast<const float4*>(s + c));
-          q[0] += (double)(a.x * a.x + a.y * a.y + a.z * a.z + a.w * a.w);
-          q[1] += (double)(b.x * b.x + b.y * b.y + b.z * b.z + b.w * b.w);
-          q[2] += (double)(a.x * b.x + a.y * b.y + a.z * b.z + a.w * b.w);
-          q[3] += (double)(e.x * e.x + e.y * e.y + e.z * e.z + e.w * e.w);
-          q[4] += (double)(a.x * e.x + a.y * e.y + a.z * e.z + a.w * e.w);
-        }
+      for (int c = lane * 4; c < p.d; c += 128) {
+        const float4 a = __ldg(reinterpret_cast<const float4*>(x + c));
+        const float4 b = __ldcg(reinterpret_cast<const float4*>(y + c)), e = __ldcg(reinterpret_cast<const float4*>(s + c));
+        q[0] += (double)(a.x * a.x + a.y * a.y + a.z * a.z + a.w * a.w);
+        q[1] += (double)(b.x * b.x + b.y * b.y + b.z * b.z + b.w * b.w);
+        q[2] += (double)(a.x * b.x + a.y * b.y + a.z * b.z + a.w * b.w);
+        q[3] += (double)(e.x * e.x + e.y * e.y + e.z * e.z + e.w * e.w);
+        q[4] += (double)(a.x * e.x + a.y * e.y + a.z * e.z + a.w * e.w);
+      }
 #pragma unroll
-        for (int k = 0; k < 5; ++k) q[k] = warp_sum_d(q[k]);
-        if (lane == 0) {
-          const double nx = fmax(sqrt(q[0]), 1e-12);
-          row_cos[r - r0] = make_double2(q[2] / (nx * fmax(sqrt(q[1]), 1e-12)), q[4] / (nx * fmax(sqrt(q[3]), 1e-12)));
-        }
+      for (int k = 0; k < 5; ++k) q[k] = warp_sum_d(q[k]);
+      if (lane == 0) {
+        const double nx = fmax(sqrt(q[0]), 1e-12);
+        row_cos[r - r0] = make_double2(q[2] / (nx * fmax(sqrt(q[1]), 1e-12)), q[4] / (nx * fmax(sqrt(q[3]), 1e-12)));
       }
-      __syncthreads();
-      for (int j = r0 / p.T + 1 + tid; j <= r1 / p.T; j += THREADS) {
-        double s_app = 0.0, s_skip = 0.0;
-        for (int t = 0; t < p.T; ++t) {
-          const double2 q = row_cos[(j - 1) * p.T - r0 + t];
-          s_app += q.x;
-          s_skip += q.y;
-        }
-        const float a = (float)(s_app / p.T), s = (float)(s_skip / p.T);
-        int take = 0;
-        const long long cell = (long long)i * (p.M + 1) + j;
-        if (j <= n) {
-          take = a > s;
-          if (p.forced && p.forced[cell] != 255) take = p.forced[cell] == 0;
-        }
-        s_take[j - 1] = take;
-        s_choice[cell] = take ? 0 : 1;
-        if (rank == 0) {
-          p.scores[cell] = take ? a : s;
-          if (p.margins && j <= n) p.margins[cell] = a - s;
-        }
-      }
-      __syncthreads();
     }
+    __syncthreads();
+    for (int j = j_lo + tid; j <= states; j += THREADS) {
+      double s_app = 0.0, s_skip = 0.0;
+      for (int t = 0; t < p.T; ++t) {
+        const double2 q = row_cos[(j - 1) * p.T - r0 + t];
+        s_app += q.x;
+        s_skip += q.y;
+      }
+      const float a = (float)(s_app / p.T), s = (float)(s_skip / p.T);
+      int take = 0;
+      const long long cell = (long long)i * (p.M + 1) + j;
+      if (j <= n) {
+        take = a > s;
+        if (p.forced && p.forced[cell] != 255) take = p.forced[cell] == 0;
+      }
+      s_take[j - 1] = take;
+      s_choice[cell] = take ? 0 : 1;
+      if (rank == 0) {
+        p.scores[cell] = take ? a : s;
+        if (p.margins && j <= n) p.margins[cell] = a - s;
+      }
+    }
+    __syncthreads();
     if (tid == 0) {
       s_choice[(long long)i * (p.M + 1)] = 0;
       if (rank == 0) p.scores[(long long)i * (p.M + 1)] = 1.0f;
     }
     __syncthreads();
-    for (int r = (j_lo - 1) * p.T + rank + warp * CTAS; r < states * p.T; r += CTAS * WARPS) {
+    for (int r = r0 + rank + warp * CTAS; r < r1; r += CTAS * WARPS) {
       const int j = r / p.T + 1, t = r % p.T;
       const float* src = s_take[j - 1] ? p.G + (long long)r * p.d : skip_row(g_prev, i, r);
       for (int c = lane * 4; c < p.d; c += 128) {
