@@ -13,7 +13,8 @@ from tests.util import Pair, close_hidden, kv_to_oracle, tol_hidden
 
 pytestmark = pytest.mark.gpu
 
-ENGINES = [("tiny", 0), ("small", 0), ("mini8b", 0)]
+FLAG_MULTI_KERNEL = 4
+ENGINES = [("tiny", 0), ("small", 0), ("mini8b", 0), ("tiny", FLAG_MULTI_KERNEL)]
 
 
 @pytest.fixture(scope="module", params=ENGINES, ids=lambda p: f"{p[0]}-flags{p[1]}")

@@ -15,9 +15,9 @@ from tests.util import Pair, check_search_against_oracle, close_hidden, kv_to_or
 pytestmark = pytest.mark.gpu
 
 FLAG_FORCE_SIMT, FLAG_NO_DEFER, FLAG_MULTI_KERNEL, FLAG_PRUNE = 1, 2, 4, 8
-# (config name, library flags): the fp32 model runs the CUDA-core GEMM; the bf16 models run
-# the tcgen05 GEMM, and once more with the CUDA-core GEMM as a cross-check of the rest.
-ENGINES = [("tiny", 0), ("small", 0), ("mini8b", 0), ("small", FLAG_FORCE_SIMT)]
+# (config name, library flags): the small fp32 model runs one cluster per call and, as larger fp32 models do, one kernel
+# per step; the bf16 models run the persistent tcgen05 kernel, and once more the CUDA-core GEMM as a cross-check of the rest.
+ENGINES = [("tiny", 0), ("small", 0), ("mini8b", 0), ("small", FLAG_FORCE_SIMT), ("tiny", FLAG_MULTI_KERNEL)]
 
 
 @pytest.fixture(scope="module", params=ENGINES, ids=lambda p: f"{p[0]}-flags{p[1]}")

@@ -1,18 +1,21 @@
 """The one-launch path of fp32 models that fit a cluster (csrc/small32.cuh) against one kernel per step
-(CLASP_FLAG_MULTI_KERNEL, itself compared with the oracle in test_gpu_parity.py): both head dimensions, widths that are no
-multiple of a warp's stride, rows around the passes of eight, ragged key blocks, an LM head that fits its slice and one
-that does not, a draft that skips every layer.
+(CLASP_FLAG_MULTI_KERNEL, which test_gpu_parity.py and test_gpu_draft_and_loop.py compare with the oracle beside it): both
+head dimensions, widths that are no multiple of a warp's stride, rows around the passes of eight, ragged key blocks, an LM
+head that fits its slice and one that does not, a draft that skips every layer.  Whole calls at head dimension 128 against
+the oracle; calls on either side of the limits of the path over one cache.
 
 Both sides sum at most 704 products in fp32 in different orders: the expected difference is about sqrt(704) * 6e-8 = 2e-6
 of a value's scale, growing over the layers; 2e-5 leaves a factor of ten."""
 import dataclasses
 
+import numpy as np
 import pytest
 import torch
 
 import datagen
 import paper_2505_24196_b200 as clasp
-from tests.util import rel_l2
+from oracle import clasp_oracle as orc
+from tests.util import Pair, check_search_against_oracle, close_hidden, rel_l2, tol_hidden
 
 pytestmark = pytest.mark.gpu
 TOL = 2e-5
@@ -28,14 +31,15 @@ MODELS = {
 class Two:
     """The same weights in a context of either path."""
 
-    def __init__(self, cfg):
+    def __init__(self, cfg, max_ctx=200, max_rows=64):
         self.cfg = cfg
         layers = [{k: v.cuda().contiguous() for k, v in datagen.layer_weights(cfg, l, "cpu").items()} for l in range(cfg.L)]
         head = {k: v.cuda().contiguous() for k, v in datagen.head_weights(cfg, "cpu").items()}
         self.layers, self.head = layers, head
         self.eng = []
         for flags in (0, clasp.FLAG_MULTI_KERNEL):
-            e = clasp.Clasp(clasp.make_config(cfg, max_ctx=200, max_rows=64, max_M=cfg.L, max_T=8, max_head_rows=16, flags=flags))
+            e = clasp.Clasp(clasp.make_config(cfg, max_ctx=max_ctx, max_rows=max_rows, max_M=cfg.L, max_T=8, max_head_rows=16,
+                                             flags=flags))
             e.load_layers(0, layers)
             e.load_head(head)
             self.eng.append(e)
@@ -183,3 +187,57 @@ def test_norm_keeps_small_columns():
     want = float(torch.rsqrt((row * row).mean() + cfg.rms_eps))
     assert abs(float(kv.v[0, 0, 0, 0]) / want - 1.0) < 2.0 ** -23
     e.close()
+
+
+@pytest.mark.parametrize("flags", [0, clasp.FLAG_MULTI_KERNEL], ids=["one-launch", "per-step"])
+def test_head_dimension_128_against_the_oracle(flags):
+    """Verification, draft and search of an fp32 model with head dimension 128 (tolerances of test_gpu_parity.py)."""
+    cfg = MODELS["hd128"]
+    p = Pair(cfg, max_ctx=96, max_rows=64, max_M=3, max_T=2, max_head_rows=4, flags=flags)
+    n, L, d, M, T = 41, cfg.L, cfg.d_model, 3, 2
+    toks = datagen.token_ids(cfg, n)
+    oc, kv = p.new_oracle_cache(), p.new_kv()
+    am_o, hid_o, logits = orc.verify_forward(p.oracle, toks.numpy(), oc, 0)
+    am, hid = p.engine.verify(toks.cuda(), 0, kv, 4)
+    assert close_hidden(hid.cpu().numpy(), hid_o, tol_hidden(cfg))
+    top = np.sort(logits[-4:], axis=-1)
+    assert (am.cpu().numpy() == am_o[-4:])[top[:, -1] - top[:, -2] > 1e-3 * np.abs(logits).max()].all()
+    p0 = n - T
+    ref = orc.dp_search(p.oracle, np.transpose(hid_o[p0:n], (1, 0, 2)), oc, p0, p0, M)
+    res = p.engine.dp_search(hid[p0], d, (L + 1) * d, kv, p0, p0, T, M)
+    D, margin, S = (res[k].cpu().numpy() for k in ("D", "margin", "S"))
+    assert np.array_equal(np.isnan(D), np.isnan(ref["D"]))
+    check_search_against_oracle(D, margin, S, res["g_final"].cpu().numpy(), ref, L, M, tol_hidden(cfg))
+    forced = torch.from_numpy(ref["choice"].copy()).cuda()
+    rf = p.engine.dp_search(hid[p0], d, (L + 1) * d, kv, p0, p0, T, M, forced_choice=forced)
+    ok = ~np.isnan(ref["D"])
+    np.testing.assert_allclose(rf["D"].cpu().numpy()[ok], ref["D"][ok], atol=1e-6)
+    assert close_hidden(rf["g_final"].cpu().numpy(), ref["g"][L, M], tol_hidden(cfg))
+    assert p.engine.device_status() == 0
+    p.engine.close()
+
+
+def test_one_cache_on_both_sides_of_the_limits():
+    """A prompt in pieces of 128, 129 and 51 rows, then verifications and single rows around the limits: 128 rows, 2048
+    positions, 65536 scores (rows x heads x keys).  The launches of a call tell its route; every piece continues the cache of
+    the one before, whichever route wrote it."""
+    cfg = dataclasses.replace(TINY, L=2)
+    two = Two(cfg, max_ctx=2100, max_rows=129)
+    caches = two.caches(0)
+    toks = datagen.token_ids(cfg, 2100).to(torch.int32).cuda()
+    pos, routes = 0, []
+    for n in [128, 129, 51] + [129] * 13 + [9, 8, 45, 1, 1, 7]:
+        keys = pos + n
+        one = n <= 128 and keys <= 2048 and n * cfg.n_q_heads * keys <= 65536
+        res = []
+        for e, kv in zip(two.eng, caches):
+            n0 = e.launch_count()
+            am, hid = e.verify(toks[pos:keys], pos, kv, 1)
+            res.append((am, hid, e.launch_count() - n0))
+            assert e.device_status() == 0
+        assert (res[0][2] == 1) == one and res[1][2] > 10, (n, keys, res[0][2])
+        assert close(res[0][1], res[1][1]) and torch.equal(res[0][0], res[1][0]), (n, keys)
+        routes.append(one)
+        pos = keys
+    assert routes == [True, False, True] + [False] * 13 + [False, True, False, True, False, False]
+    assert close(caches[0].k[:, :pos], caches[1].k[:, :pos]) and close(caches[0].v[:, :pos], caches[1].v[:, :pos])
