@@ -133,14 +133,19 @@ int clasp_create(const clasp_config* cfg, void* workspace, size_t workspace_byte
                  void* cuda_stream, clasp_ctx** out);
 void clasp_destroy(clasp_ctx* ctx);
 
-/* 1 when the context runs its searches and forwards in the persistent layer kernel (one
- * cooperative launch per call), 0 when it uses one kernel per step: an fp32 model, the two
- * diagnostic flags above, or a bf16 shape the persistent kernel does not take (vocab not a
- * multiple of 8; more than 128 d_model features per SM; a weight matrix whose per-SM row
- * ranges need more than four distinct heights; no cooperative launch on the device).  Both
- * paths compute the same thing; the second is several times slower, so a caller that sized
- * its deployment for the first should check.  Per call, a search with M*T > 128 candidate
- * rows and a forward over more than 128 rows also take the one-kernel-per-step path.
+/* 1 when the context runs its searches and forwards in the persistent layer kernel (bf16
+ * models: one cooperative launch per call), 0 otherwise: any fp32 model, a bf16 model with
+ * one of the two diagnostic flags above, or a bf16 shape the persistent kernel does not take
+ * (vocab not a multiple of 8; more than 128 d_model features per SM; a weight matrix whose
+ * per-SM row ranges need more than four distinct heights; no cooperative launch on the
+ * device).  Such a bf16 context runs one kernel per step: the same thing, several times
+ * slower, so a caller that sized its deployment for the other path should check.  Per call,
+ * a search with M*T > 128 candidate rows and a forward over more than 128 rows run one kernel
+ * per step in any case.
+ * fp32 models read 0 either way: one whose layer fits the shared memory of sixteen CTAs (L at
+ * most 32, max_M at most 63, a layer of up to about 3 MB) runs a call of up to 128 rows, 2048
+ * positions and 65536 scores (rows x query heads x positions) in one launch of its own kernel
+ * -- clasp_launch_count tells --, anything else in one kernel per step.
  * Negative: CLASP_ERR_INVALID_ARG. */
 int clasp_engine_active(const clasp_ctx* ctx);
 

@@ -1,6 +1,8 @@
 // C ABI of the layer-skip search library: context, argument checks and the host-side
-// launch sequences.  Every arithmetic step runs in the kernels of kernels.cuh and
-// gemm_tc.cuh; this file only sequences launches on the caller's stream.
+// launch sequences.  Every arithmetic step runs in a kernel -- engine2.cuh (bf16 calls of up
+// to 128 rows), wide.cuh (bf16 layers over more), small32.cuh (calls on small fp32 models),
+// kernels.cuh and gemm_tc.cuh (one kernel per step: everything else), sampling.cuh --; this
+// file only sequences launches on the caller's stream.
 #include "../../include/clasp.h"
 
 #include <cuda.h>
@@ -433,12 +435,21 @@ int gemm_wide(clasp_ctx* ctx, const GemmCall& g) {
     f_tiles += p.f_tiles[m];
   }
   p.tiles = f_tiles * p.row_tiles;
-  // pairs at work: one per two SMs, each with at least a handful of chunks
+  // Pairs at work: one per two SMs, each with at least eight chunks.  Four chunks make the small products slower (down
+  // product of d_ffn 3584, 129 - 500 rows: 50 us against 39), sixteen faster (34 - 37; o product of the 8B shape, 129 rows,
+  // 35 against 43, the other 8B products the same).
   int W = ctx->num_sms / 2;
   const long long units = (long long)p.tiles * p.kc;
   if (units / 8 < W) W = units / 8 < 1 ? 1 : (int)(units / 8);
   // What whole waves of tiles leave over is split over K, together with one whole wave (a tile then has two or three
-  // parts); a last wave that is at least 15/16 full stays whole.
+  // parts); a last wave that is at least 15/16 full stays whole.  Single launches on the 8B shape, us, as split here / the
+  // left-over tiles alone split / nothing split:
+  //    257 rows   q/k/v  45 /  44 /  33   o  43 /  43 /  35   gate/up 109 / 215 / 105   down  71 /  72 /  84
+  //   1300 rows          60 /  60 /  60      71 /  66 /  60           232 / 271 / 236        174 / 136 / 173
+  //   1999 rows          91 /  90 /  89      86 /  74 /  68           307 / 333 / 314        247 / 183 / 193
+  // So splitting pays for down products of a few row tiles; past those the partial sums (up to 38 MB written and read back
+  // per product) cost more than the uneven last wave they fill.  A limit of 7/8 instead of 15/16 changes nothing at these
+  // sizes; without one the q/k/v product of 1300 rows (70 of 74 pairs in its last wave) takes 75 us instead of 60.
   const int full = p.tiles / W, left = p.tiles - full * W;
   p.sk_tiles = left == 0 || (W - left) * 16 <= W ? 0 : left + (full > 0 ? W : 0);
   if (p.sk_tiles * 2 > MAX_COUNTERS || (size_t)W * 4 * wd::SLOT_FLOATS > PARTIAL_FLOATS) p.sk_tiles = 0;
@@ -780,8 +791,9 @@ int s32_forward(clasp_ctx* ctx, s32::Params* p, const int32_t* tokens, int n, fl
 // ---------------------------------------------------------------- persistent layer engine
 // Host side of engine2.cuh: builds the job list of a call and launches the cooperative
 // kernel once.  Used by the bf16 tensor-core configuration; the per-kernel sequences
-// above remain for the fp32 model, for CLASP_FLAG_FORCE_SIMT and for shapes the engine
-// does not take (more than 128 rows).
+// above remain for fp32 models beyond small32.cuh, for CLASP_FLAG_FORCE_SIMT and
+// CLASP_FLAG_MULTI_KERNEL and for what the engine does not take (more than 128 rows, whose
+// products and attention are those of wide.cuh).
 namespace pk = clasp::pk;
 
 int engine_setup(clasp_ctx* ctx) {

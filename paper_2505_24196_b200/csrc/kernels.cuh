@@ -2,8 +2,8 @@
 // is not a weight-streaming GEMM on the tensor cores (RMSNorm, rotary embedding,
 // attention over the verified cache plus a state's own rows, the cosine / select /
 // write-back step of Eq. 2, the backtrack of Algorithm 1, embedding gather, argmax),
-// plus a CUDA-core GEMM used by the fp32 model (whose tolerance rules out bf16
-// tensor-core products).
+// plus a CUDA-core GEMM for fp32 models (whose tolerance rules out bf16 tensor-core
+// products).  One kernel per step; small fp32 models run a call in one launch (small32.cuh).
 #pragma once
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>

@@ -6,7 +6,7 @@
 // ramp, tail), here a step ends in a hardware cluster barrier.  Every CTA owns a slice of each matrix's output features;
 // its slices of the next layer are on their way to shared memory (bulk copies) while the current one is multiplied.
 // Activations cross between the CTAs through global memory (L2).
-// Measured on 256 columns, 8 layers: search over 64 positions 396 -> 148 us, draft token 310 -> 108, verification of five
+// Measured on 256 columns, 8 layers: search over 64 positions 396 -> 146 us, draft token 310 -> 108, verification of five
 // rows 474 -> 176.  A layer takes about 15 us: five hand-offs of about 2000 cycles (stores to L2 before the barrier, the
 // barrier, loads from L2 behind it) and as much again for what the 16 SMs read from shared memory and shuffle.
 #pragma once

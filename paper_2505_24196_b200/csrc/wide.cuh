@@ -223,12 +223,14 @@ __device__ __forceinline__ bool epi_any(bool p) {
 
 // y[r, n] = sum_k x[r, k] w[n, k] over tiles of 256 rows x 256 features (SwiGLU: 128 gate and 128 up features).  A pair
 // of CTAs multiplies a tile: each loads 128 rows of x and 128 rows of W, the even CTA issues M = 256 MMAs that read
-// both, each keeps the accumulator of its own 128 rows.  Bound: tensor cores; a 64-column chunk is 512 cycles of
-// multiplies for 32 KB of loads per SM (one CTA per tile of 128 x 256 would need 48 KB for the same work).  Measured, 8B
-// shape, 1999 rows: 702 us for the four products of a layer = 1.24 PFLOP/s in a single pass; under the power cap of a loop
-// about 1.0.  (Passes of 256 rows through the skinny product, which re-read all weights eight times, and the CUDA-core
-// attention took 14.9 ms per layer together.)  At 128 rows the four products take 216 us against 114 inside the persistent
-// kernel (partial sums of the split tiles, ramps), so that kernel keeps the launches of up to 128 rows.
+// both, each keeps the accumulator of its own 128 rows.  A 64-column chunk is 512 cycles of multiplies for 32 KB of loads
+// per SM (one CTA per tile of 128 x 256 would need 48 KB for the same work).  Measured, 8B shape, 1999 rows, PFLOP/s in a
+// loop under the power cap, a plain library product of the same shape beside it: gate/up 1.21 / 1.25, q/k/v 0.99 / 1.27, o
+// 0.78 / 1.28, down 0.79 / 1.32 (single launches 1.25, 1.20, 0.65 - 0.78, 0.85 - 0.95).  Gate/up is bound by the tensor
+// cores; the others lose a quarter and more to the partial sums of their split tiles.  (Passes of 256 rows through the
+// skinny product, which re-read all weights eight times, and the CUDA-core attention took 14.9 ms per layer together.)  At
+// 128 rows the four products take 216 us against 114 inside the persistent kernel (partial sums, ramps), so that kernel
+// keeps the launches of up to 128 rows.
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS, 1)
 gemm_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w0,
             const __grid_constant__ CUtensorMap map_w1, const __grid_constant__ CUtensorMap map_w2, const GemmParams p) {
@@ -531,8 +533,10 @@ __device__ __forceinline__ void split2(float x, float y, uint32_t& hi, uint32_t&
 // Attention of the rows' queries over the cache keys [0, C) and the own rows (row r sees own rows of its state, of T
 // rows, up to itself).  A CTA takes ATT_PAIRS pairs (row, query head) of one kv head through its key tiles:
 //   S = Q K^T, softmax weights P = exp2(S - m), O += P V, all multiplies on tcgen05, S / P / O in tensor memory.
-// Queries and weights keep 16 mantissa bits: both enter their product as a bf16 pair (high + low part), two multiplies
-// each.  A thread owns a pair; its maximum m moves only when exceeded by more than 2^8 (then O is rescaled).
+// Queries and weights enter their product as a bf16 pair each (high + low part, two multiplies): 17 bits where the attention
+// on the CUDA cores held 24.  What that leaves is far below the rounding of the result to the bf16 operand of the o
+// projection: error of the attention alone against float64, weights that cancel, 1.6457e-3 - 1.6621e-3 with fp32 operands'
+// 1.6454e-3 - 1.6619e-3 beside it, of 52 prompts of 129 - 1000 rows 0.9999 +- 0.0002 times as large.  A thread owns a pair; its maximum m moves only when exceeded by more than 2^8 (then O is rescaled).
 // Scores are double-buffered so that the next tile's Q K^T runs under this tile's softmax, and two CTAs share an SM.
 // Bound by the multiplies (four per score and value because of the two parts): 84 us per layer at 1999 rows, 32 query
 // heads, where the tensor pipe alone needs about 30.
