@@ -1622,9 +1622,12 @@ int clasp_draft_sample(clasp_ctx* ctx, const uint8_t* skip_mask_host, const int3
   int rc = draft_impl(ctx, skip_mask_host, token_in, pos, kv, token_out, nullptr, logits_out);
   if (rc) return rc;
   // the drafted token will sit at position pos + 1
-  clasp::smp::gumbel_argmax_kernel<<<1, clasp::smp::THREADS, 0, ctx->stream>>>(
+  const int n_chunks = clasp::smp::chunks_of(ctx->cfg.vocab);
+  clasp::smp::gumbel_argmax_kernel<<<n_chunks, clasp::smp::THREADS, 0, ctx->stream>>>(
       logits_out, ctx->cfg.vocab, 1.0f / temperature, (unsigned long long)seed, pos + 1, clasp::smp::DRAW_DRAFT, round,
-      token_out);
+      ctx->ws.spec);
+  if ((rc = launch_check(ctx))) return rc;
+  clasp::smp::gumbel_merge_kernel<<<1, 32, 0, ctx->stream>>>(ctx->ws.spec, n_chunks, token_out);
   return launch_check(ctx);
 }
 
@@ -1639,13 +1642,21 @@ int clasp_verify_sample(clasp_ctx* ctx, const int32_t* tokens, int32_t n, int32_
   int rc = verify_impl(ctx, tokens, n, pos0, kv, n_drafts + 1, committed_out, hidden_out, logits_ws);
   if (rc) return rc;
   const int first = pos0 + n - n_drafts;   // position of the first draft (of the sampled token when there is none)
-  clasp::smp::spec_rows_kernel<<<n_drafts + 1, clasp::smp::THREADS, 0, ctx->stream>>>(
-      logits_ws, draft_logits, tokens + (n - n_drafts), n_drafts, ctx->cfg.vocab, 1.0f / temperature,
-      (unsigned long long)seed, first, round, ctx->ws.spec);
+  const int n_chunks = clasp::smp::chunks_of(ctx->cfg.vocab), vocab = ctx->cfg.vocab;
+  const float inv_t = 1.0f / temperature;
+  const int32_t* drafts = tokens + (n - n_drafts);
+  clasp::smp::spec_norm_kernel<<<dim3(n_chunks, n_drafts + 1), clasp::smp::THREADS, 0, ctx->stream>>>(
+      logits_ws, draft_logits, n_drafts, vocab, inv_t, (unsigned long long)seed, first, round, ctx->ws.spec);
   if ((rc = launch_check(ctx))) return rc;
-  clasp::smp::spec_commit_kernel<<<1, 32, 0, ctx->stream>>>(ctx->ws.spec, tokens + (n - n_drafts), n_drafts,
-                                                            (unsigned long long)seed, first, round, n_accepted_out,
-                                                            committed_out);
+  if (n_drafts > 0) {
+    clasp::smp::spec_rows_kernel<<<dim3(n_chunks, n_drafts), clasp::smp::THREADS, 0, ctx->stream>>>(
+        logits_ws, draft_logits, vocab, inv_t, (unsigned long long)seed, first, round, ctx->ws.spec);
+    if ((rc = launch_check(ctx))) return rc;
+  }
+  clasp::smp::spec_commit_kernel<<<1, clasp::smp::THREADS, 0, ctx->stream>>>(ctx->ws.spec, logits_ws, draft_logits, drafts,
+                                                                             n_drafts, n_chunks, vocab, inv_t,
+                                                                             (unsigned long long)seed, first, round,
+                                                                             n_accepted_out, committed_out);
   return launch_check(ctx);
 }
 
