@@ -162,3 +162,43 @@ def test_committed_token_is_distributed_as_the_full_model(pair, T):
     assert ok, stat
     rate = float(np.minimum(p0, q0).sum())
     assert abs(accepted / N - rate) < 5 * math.sqrt(max(rate * (1 - rate), 1e-4) / N) + 1e-3
+
+
+@pytest.mark.parametrize("vocab", [40, 2048, 2056, 16640, 131072, 133000])
+def test_rows_cut_into_parts(vocab):
+    """A row of logits is drawn in up to 64 parts of 256 k values: vocabularies of less than one part, one whole part, a
+    ragged second one, a multiple of the stride, 64 full parts and more than 64 x 2048 values; drafts from a model that gives all
+    but five tokens no weight at all (whole parts of -inf)."""
+    import dataclasses
+    import paper_2505_24196_b200 as clasp
+    cfg = dataclasses.replace(datagen.CONFIGS["tiny"], L=1, d_model=64, n_q_heads=1, n_kv_heads=1, d_ffn=64, vocab=vocab)
+    eng = clasp.Clasp(clasp.make_config(cfg, max_ctx=32, max_rows=8, max_M=1, max_head_rows=4))
+    eng.load_layers(0, [datagen.layer_weights(cfg, 0, "cuda")])
+    eng.load_head(datagen.head_weights(cfg, "cuda"))
+    kv = clasp.KVCache(eng.cfg)
+    K, n, T = 2, 4, 0.7
+    bufs = _buffers(cfg, K)
+    tok, q, p, n_acc, committed = bufs
+    eng.verify(datagen.token_ids(cfg, n).cuda().int(), 0, kv, 0, want_hidden=False)
+    wrong = 0
+    for trial in range(8):
+        seed = 77 + trial
+        tok[:1] = trial
+        for k in range(K):
+            eng.draft_sample(bytes(1), tok[k:k + 1], n + k, kv, T, seed, 1, tok[k + 1:k + 2], q[k])
+        drafts = tok[1:].cpu().tolist()
+        q64 = q.double().cpu().numpy()
+        wrong += sum(d != orc.gumbel_max_sample(q64[k], T, seed, n + k + 1, orc.DRAW_DRAFT, 1) for k, d in enumerate(drafts))
+        if trial % 2:
+            keep = torch.tensor(drafts + [0, vocab // 2, vocab - 1], device="cuda")
+            mask = torch.full_like(q, -math.inf)
+            mask[:, keep] = 0.0
+            q += mask
+            q64 = q.double().cpu().numpy()
+        eng.verify_sample(tok, n, kv, K, q, T, seed, 1, p, n_acc, committed)
+        torch.cuda.synchronize()
+        a = int(n_acc[0])
+        a_o, new_o = orc.speculative_accept(p.double().cpu().numpy(), q64, drafts, T, seed, n + 1, 1)
+        wrong += (a, committed[:a + 1].cpu().tolist()) != (a_o, new_o)
+    assert wrong <= 1 and eng.device_status() == 0     # (a float near-tie may flip one of 24 decisions)
+    eng.close()
