@@ -441,17 +441,17 @@ int gemm_wide(clasp_ctx* ctx, const GemmCall& g) {
   int W = ctx->num_sms / 2;
   const long long units = (long long)p.tiles * p.kc;
   if (units / 8 < W) W = units / 8 < 1 ? 1 : (int)(units / 8);
-  // What whole waves of tiles leave over is split over K, together with one whole wave (a tile then has two or three
-  // parts); a last wave that is at least 15/16 full stays whole.  Single launches on the 8B shape, us, as split here / the
-  // left-over tiles alone split / nothing split:
-  //    257 rows   q/k/v  45 /  44 /  33   o  43 /  43 /  35   gate/up 109 / 215 / 105   down  71 /  72 /  84
-  //   1300 rows          60 /  60 /  60      71 /  66 /  60           232 / 271 / 236        174 / 136 / 173
-  //   1999 rows          91 /  90 /  89      86 /  74 /  68           307 / 333 / 314        247 / 183 / 193
-  // So splitting pays for down products of a few row tiles; past those the partial sums (up to 38 MB written and read back
-  // per product) cost more than the uneven last wave they fill.  A limit of 7/8 instead of 15/16 changes nothing at these
-  // sizes; without one the q/k/v product of 1300 rows (70 of 74 pairs in its last wave) takes 75 us instead of 60.
+  // What whole waves of tiles leave over is split over K where that saves a pair at least SPLIT_MIN_SAVED chunks: a chunk
+  // takes 0.27 - 0.31 us, the partial sums of a split tile (131 KB per part and CTA, written, counted and read back) 16 us
+  // and 0.1 us per chunk.  Single launches on the 8B shape, us, left-over tiles split / together with one whole wave / nothing:
+  //    257 rows   q/k/v  44 /  45 /  33   o  43 /  43 /  35   gate/up 215 / 109 / 105   down  72 /  71 /  84
+  //   1300 rows          60 /  60 /  60      66 /  71 /  60           271 / 232 / 236        136 / 174 / 173
+  //   1999 rows          90 /  91 /  89      74 /  86 /  68           333 / 307 / 314        183 / 247 / 193
+  // and 1999 rows in a loop under the power cap 99 / 102 / 95, 81 / 86 / 71, 409 / 388 / 386, 219 / 299 / 213.  So it pays
+  // for down products whose last wave is up to half full (257 rows save 127 chunks, 1300 rows 157; 1999 rows would save 60).
+  constexpr int SPLIT_MIN_SAVED = 100;
   const int full = p.tiles / W, left = p.tiles - full * W;
-  p.sk_tiles = left == 0 || (W - left) * 16 <= W ? 0 : left + (full > 0 ? W : 0);
+  p.sk_tiles = left > 0 && p.kc - (int)((long long)left * p.kc / W) >= SPLIT_MIN_SAVED ? left : 0;
   if (p.sk_tiles * 2 > MAX_COUNTERS || (size_t)W * 4 * wd::SLOT_FLOATS > PARTIAL_FLOATS) p.sk_tiles = 0;
   p.epi = g.epi;
   p.yf = g.yf; p.ldy = g.ldy; p.resid = g.resid; p.ldr = g.ldr; p.yo = (bf16*)g.yo; p.ldo = g.ldo;

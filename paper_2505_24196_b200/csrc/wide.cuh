@@ -164,8 +164,7 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32
 
 // ------------------------------------------------------------------ the products
 // Work list of a pair w of W: first its share of the tiles that are split over K -- all their (tile, chunk) units in one
-// row, cut into W equal ranges --, then whole tiles w, w + W, ...  The split part is what whole waves of tiles leave
-// over, so every pair has the same number of chunks to multiply.
+// row, cut into W equal ranges --, then whole tiles w, w + W, ...  The split part, if any, is what whole waves of tiles leave over.
 struct Items {
   long long u, u1;
   int dp, W;
@@ -225,10 +224,10 @@ __device__ __forceinline__ bool epi_any(bool p) {
 // of CTAs multiplies a tile: each loads 128 rows of x and 128 rows of W, the even CTA issues M = 256 MMAs that read
 // both, each keeps the accumulator of its own 128 rows.  A 64-column chunk is 512 cycles of multiplies for 32 KB of loads
 // per SM (one CTA per tile of 128 x 256 would need 48 KB for the same work).  Measured, 8B shape, 1999 rows, PFLOP/s in a
-// loop under the power cap, a plain library product of the same shape beside it: gate/up 1.21 / 1.25, q/k/v 0.99 / 1.27, o
-// 0.78 / 1.28, down 0.79 / 1.32 (single launches 1.25, 1.20, 0.65 - 0.78, 0.85 - 0.95).  Gate/up is bound by the tensor
-// cores; the others lose a quarter and more to the partial sums of their split tiles.  (Passes of 256 rows through the
-// skinny product, which re-read all weights eight times, and the CUDA-core attention took 14.9 ms per layer together.)  At
+// loop under the power cap, a plain library product of the same shape beside it: gate/up 1.22 / 1.25, q/k/v 1.06 / 1.27, o
+// 0.94 / 1.28, down 1.11 / 1.32.  All four read about 11 TB/s from L2 into shared memory; gate/up is at the power cap beside.
+// (Passes of 256 rows through the skinny product, which re-read all weights eight times, and the CUDA-core attention took
+// 14.9 ms per layer together.)  At
 // 128 rows the four products take 216 us against 114 inside the persistent kernel (partial sums, ramps), so that kernel
 // keeps the launches of up to 128 rows.
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS, 1)

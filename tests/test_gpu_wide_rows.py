@@ -101,11 +101,11 @@ def test_products_are_in_the_launch_timing(pair):
 
 # (model, rows, states): what the 74 pairs of CTAs do with the 256-row tiles of q/k/v, o, gate/up and down
 SCHEDULES = [
-    ("mini8b", 1999, 1999),   # gate/up: 224 tiles, 76 of them split (ranges over two tiles), then two whole ones per pair; rest split
-    ("mini8b", 1300, 26),     # gate/up: 168 tiles, 94 split, one whole per pair
-    ("small", 1999, 1999),    # gate/up: all 88 tiles split over 74 pairs; q/k/v and o one whole tile per pair
-    ("8b", 129, 43),          # gate/up: all 112 tiles split over 74 pairs; rest split
-    ("8b", 1300, 260),        # q/k/v: 144 whole tiles, the last wave short of four; gate/up: 80 of 672 split, then eight per pair
+    ("mini8b", 1999, 1999),   # gate/up: 224 tiles, up to four per pair; nothing split (few chunks of K)
+    ("mini8b", 1300, 26),     # gate/up: 168 tiles
+    ("small", 1999, 1999),    # gate/up: 88 tiles on 74 pairs; q/k/v and o one per pair at most
+    ("8b", 129, 43),          # down: all 16 tiles split over 74 pairs; the others whole
+    ("8b", 1300, 260),        # down: 22 of 96 tiles split, then one whole tile per pair
 ]
 
 
