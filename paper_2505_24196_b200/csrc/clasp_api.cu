@@ -943,6 +943,29 @@ double job_bytes(const clasp_ctx* ctx, const pk::Job& J) {
   return 2.0 * (d * (qd + 2 * kvd) + qd * d + 3.0 * d * c.d_ffn) + 2.0 * (double)J.C * kvd * 2.0;
 }
 
+template <int N>
+int setup_launch_n(clasp_ctx* ctx, clasp::SetupArgs& a, size_t bytes) {
+  clasp::JobList<N> list;
+  if (bytes <= sizeof(list)) {
+    memcpy(&list, ctx->e_jobs.data(), bytes);
+    a.n_jobs16 = (int)((bytes + 15) / 16);
+  }
+  clasp::setup_kernel<N><<<ctx->e_G, 256, 0, ctx->stream>>>(a, list);
+  return launch_check(ctx);
+}
+// The set-up kernel in front of the engine, with the job list as its parameter (a list beyond 31 KB is copied instead).
+int setup_launch(clasp_ctx* ctx, clasp::SetupArgs a) {
+  const size_t bytes = ctx->e_jobs.size() * sizeof(pk::Job);
+  static_assert(sizeof(pk::Job) % 16 == 0, "the list is copied in 16-byte pieces");
+  a.jobs = (uint4*)ctx->ws.jobs;
+  a.n_jobs16 = 0;
+  if (bytes <= sizeof(clasp::JobList<128>)) return setup_launch_n<128>(ctx, a, bytes);
+  if (bytes <= sizeof(clasp::JobList<768>)) return setup_launch_n<768>(ctx, a, bytes);
+  if (bytes <= sizeof(clasp::JobList<1984>)) return setup_launch_n<1984>(ctx, a, bytes);
+  CUDA_TRY(cudaMemcpyAsync(ctx->ws.jobs, ctx->e_jobs.data(), bytes, cudaMemcpyHostToDevice, ctx->stream));
+  return setup_launch_n<128>(ctx, a, bytes);
+}
+
 // Launch the engine over ctx->e_jobs.  Rmax: most rows of any job; head_off: first row of the
 // previous job that the head job (if any) reads.
 // `setup`: rotary table and the call's own tables or embedded rows; the rest of it is filled in here.
@@ -1050,14 +1073,11 @@ int engine_launch(clasp_ctx* ctx, int Rmax, int head_off, clasp::SetupArgs setup
     CUDA_TRY(cudaMemcpyAsync(ws.kvmaps, ctx->e_kvmaps_host.data(), ctx->e_kvmaps_host.size() * sizeof(CUtensorMap),
                              cudaMemcpyHostToDevice, ctx->stream));
   }
-  CUDA_TRY(cudaMemcpyAsync(ws.jobs, ctx->e_jobs.data(), ctx->e_jobs.size() * sizeof(pk::Job),
-                           cudaMemcpyHostToDevice, ctx->stream));
   setup.abort = &ws.ctl->abort;   // (the status word is sticky)
   setup.zero = (uint4*)ws.ss_a; setup.n_zero = (int)(ws.acc_bytes / 16);   // all fixed-point accumulators
   setup.flags = ws.flags; setup.n_flags = pk::N_FLAGS * (ctx->e_G + 32);
-  clasp::setup_kernel<<<ctx->e_G, 256, 0, ctx->stream>>>(setup);
   {
-    const int rc = launch_check(ctx);
+    const int rc = setup_launch(ctx, setup);
     if (rc) return rc;
   }
 
@@ -1366,8 +1386,10 @@ int clasp_dp_search(clasp_ctx* ctx, const float* hidden_states, int64_t layer_st
     // one cooperative launch for the whole search: step i = (layer i-1 over the candidate
     // states) + (Eq. 2 select); row 0 of the g table is x_i itself and is never stored
     ctx->e_jobs.clear();
-    int cur = 0, prev_lo = 1;
-    for (int i = 1; i <= L; ++i) {
+    // (step 1 decides nothing: the set-up kernel fills its cell and leaves x_0 as g[1][1]; a model of one layer has no other)
+    const bool first = L > 1;
+    int cur = first ? 1 : 0, prev_lo = 1;
+    for (int i = first ? 2 : 1; i <= L; ++i) {
       const int ell = (i - 1 < M) ? i - 1 : M;
       // states the step carries: j_lo..ell (plus the diagonal state i while i <= M).  With pruning the
       // states from which (L, M) cannot be reached any more, j < M - (L - i), are left out; the job
@@ -1379,6 +1401,7 @@ int clasp_dp_search(clasp_ctx* ctx, const float* hidden_states, int64_t layer_st
       if (n > 0) {
         J = layer_job(ctx, i - 1, n, T, ctx_len, false, kv[i - 1]);
         J.x_in = ws.grow[cur] + j_lo * Td; J.ldx = d; J.dp = 1;
+        J.prep = ctx->e_jobs.empty() ? 1 : 0;
       } else {
         J.type = pk::JOB_SELECT; J.T = T;
       }
@@ -1413,8 +1436,13 @@ int clasp_dp_search(clasp_ctx* ctx, const float* hidden_states, int64_t layer_st
     link_jobs(ctx->e_jobs);
     clasp::SetupArgs setup = setup_args(ctx, T, pos0);
     setup.D = scores; setup.margin = margins; setup.choice = ws.choice; setup.n_cells = ncell;
+    if (first) {
+      setup.first_rows = T; setup.first_d = d; setup.first_cell = M + 1;
+      setup.x0 = hidden_states; setup.x1 = hidden_states + layer_stride; setup.x_stride = token_stride;
+      setup.g11 = ws.grow[1] + Td;
+    }
     if ((rc = engine_launch(ctx, M * T, 0, setup, ctx_len))) return rc;
-    clasp::backtrack_kernel<<<1, 32, 0, ctx->stream>>>(ws.choice, L, M, skip_mask);
+    clasp::backtrack_kernel<<<1, 256, 0, ctx->stream>>>(ws.choice, L, M, skip_mask);
     return launch_check(ctx);
   }
   clasp::fill_tables_kernel<<<(ncell + 255) / 256, 256, 0, ctx->stream>>>(scores, margins, ws.choice, ncell);
@@ -1456,7 +1484,7 @@ int clasp_dp_search(clasp_ctx* ctx, const float* hidden_states, int64_t layer_st
     if ((rc = launch_check(ctx))) return rc;
     cur ^= 1;
   }
-  clasp::backtrack_kernel<<<1, 32, 0, ctx->stream>>>(ws.choice, L, M, skip_mask);
+  clasp::backtrack_kernel<<<1, 256, 0, ctx->stream>>>(ws.choice, L, M, skip_mask);
   if ((rc = launch_check(ctx))) return rc;
   if (g_final) {
     clasp::copy_rows_kernel<<<T, 256, 0, ctx->stream>>>(ws.grow[cur] + (int64_t)M * Td, d, g_final, d, d);

@@ -492,12 +492,21 @@ __global__ void dp_step_kernel(DpStepArgs a) {
 }
 
 // Backtrack of Algorithm 1 on the choice table [(L+1) x (M+1)]: one thread.
-__global__ void backtrack_kernel(const uint8_t* __restrict__ choice, int L, int M, uint8_t* __restrict__ S) {
-  if (blockIdx.x != 0 || threadIdx.x != 0) return;
-  for (int l = 0; l < L; ++l) S[l] = 0;
+// (the table goes to shared memory first, as far as it fits: the walk is a chain of dependent reads)
+constexpr int BACKTRACK_CELLS = 16384;
+__global__ void __launch_bounds__(256) backtrack_kernel(const uint8_t* __restrict__ choice, int L, int M, uint8_t* __restrict__ S) {
+  __shared__ uint8_t cell[BACKTRACK_CELLS];
+  const int n = (L + 1) * (M + 1);
+  const bool fits = n <= BACKTRACK_CELLS;
+  if (fits)
+    for (int k = threadIdx.x; k < n; k += blockDim.x) cell[k] = choice[k];
+  for (int l = threadIdx.x; l < L; l += blockDim.x) S[l] = 0;
+  __syncthreads();
+  if (threadIdx.x != 0) return;
   int i = L, j = M;
   while (i > 0 && j > 0) {
-    if (choice[i * (M + 1) + j] == 1) {
+    const int at = i * (M + 1) + j;
+    if ((fits ? cell[at] : choice[at]) == 1) {
       S[i - 1] = 1;
       --j;
     }
@@ -590,6 +599,13 @@ struct SetupArgs {
   float* margin;
   uint8_t* choice;
   int n_cells;
+  // search: step 1 of Eq. 2.  It has one cell, the forced skip of layer 0 (no state has gone through a layer), so nothing is
+  // decided: g[1][1] = x_0, D(1, 1) = mean cos(x_1, x_0), choice (1, 1) = skip, and the kernel starts with step 2.
+  // (first_rows == 0: the step is in the job list)
+  int first_rows, first_d, first_cell;   // rows T of x_0 and x_1; columns; index of the cell (1, 0)
+  const float *x0, *x1;
+  int64_t x_stride;
+  float* g11;
   const int32_t* tokens; // forward: n_tokens rows of the table into out
   const __nv_bfloat16* table;
   int n_tokens, d, vocab;
@@ -600,10 +616,20 @@ struct SetupArgs {
   int* flags;
   int n_flags;
   int* abort;
+  uint4* jobs;           // n_jobs16 16-byte pieces of the job list, from the launch's parameters
+  int n_jobs16;
+};
+// The job list travels as a kernel parameter: a copy from pageable memory ahead of the launch is a stream operation of its
+// own that the launch waits for.  Three sizes, as a launch carries all of its parameter's bytes.
+template <int N>
+struct JobList {
+  uint4 v[N];
 };
 
-__global__ void __launch_bounds__(256) setup_kernel(const SetupArgs a) {
+template <int N>
+__global__ void __launch_bounds__(256) setup_kernel(const __grid_constant__ SetupArgs a, const __grid_constant__ JobList<N> list) {
   const int tid = blockIdx.x * blockDim.x + threadIdx.x, n = gridDim.x * blockDim.x;
+  for (int k = tid; k < a.n_jobs16; k += n) a.jobs[k] = list.v[k];
   // (the rotary table first: its double arithmetic is the longest chain; from the last block downwards, where the other
   // jobs have least to do)
   for (int k = n - 1 - tid; k < a.T * a.half; k += n) a.cs[k] = rope_entry(k, a.half, a.pos0, a.theta);
@@ -620,10 +646,49 @@ __global__ void __launch_bounds__(256) setup_kernel(const SetupArgs a) {
     }
   }
   for (int k = tid; k < a.n_cells; k += n) {
-    const float v = k == 0 ? 1.0f : __int_as_float(0x7fc00000);   // D(0, 0) = 1 (g[0][0] = x_0)
-    a.D[k] = v;
+    const bool one = k == 0 || (a.first_rows > 0 && k == a.first_cell);   // D(0, 0) = 1 (g[0][0] = x_0), D(1, 0) = 1
     if (a.margin) a.margin[k] = __int_as_float(0x7fc00000);
-    a.choice[k] = k == 0 ? 0 : 255;
+    if (a.first_rows > 0 && k == a.first_cell + 1) continue;
+    a.D[k] = one ? 1.0f : __int_as_float(0x7fc00000);
+    a.choice[k] = one ? 0 : 255;
+  }
+  if (a.first_rows > 0) {
+    for (int r = blockIdx.x; r < a.first_rows; r += gridDim.x)
+      for (int c = threadIdx.x * 4; c < a.first_d; c += blockDim.x * 4)
+        *reinterpret_cast<float4*>(a.g11 + (int64_t)r * a.first_d + c) = *reinterpret_cast<const float4*>(a.x0 + r * a.x_stride + c);
+    if (blockIdx.x == gridDim.x / 2) {   // (a block with little else to do)
+      __shared__ double part[3][8];
+      const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+      float mean = 0.f;
+      for (int t = 0; t < a.first_rows; ++t) {
+        double q[3] = {0.0, 0.0, 0.0};   // x.s, s.s, x.x with x = x_1[t], s = x_0[t]
+        for (int c = threadIdx.x * 4; c < a.first_d; c += blockDim.x * 4) {
+          const float4 u = *reinterpret_cast<const float4*>(a.x1 + t * a.x_stride + c);
+          const float4 v = *reinterpret_cast<const float4*>(a.x0 + t * a.x_stride + c);
+          q[0] += (double)(u.x * v.x + u.y * v.y + u.z * v.z + u.w * v.w);
+          q[1] += (double)(v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w);
+          q[2] += (double)(u.x * u.x + u.y * u.y + u.z * u.z + u.w * u.w);
+        }
+#pragma unroll
+        for (int e = 0; e < 3; ++e) {
+          q[e] = warp_sum_d(q[e]);
+          if (lane == 0) part[e][warp] = q[e];
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+          double v[3] = {0.0, 0.0, 0.0};
+          for (int w = 0; w < 8; ++w)
+            for (int e = 0; e < 3; ++e) v[e] += part[e][w];
+          const float nx = fmaxf(sqrtf((float)v[2]), 1e-12f);
+          mean += (float)v[0] / (nx * fmaxf(sqrtf((float)v[1]), 1e-12f));
+        }
+        __syncthreads();
+      }
+      if (threadIdx.x == 0) {
+        a.D[a.first_cell + 1] = mean / (float)a.first_rows;
+        a.choice[a.first_cell + 1] = 1;
+      }
+    }
   }
   for (int k = tid; k < a.n_zero; k += n) a.zero[k] = make_uint4(0, 0, 0, 0);
   for (int k = tid; k < a.n_flags; k += n) a.flags[k] = 0;

@@ -166,7 +166,7 @@ def cmd_trace(args):
         if len(col):
             col = (col - base) / 1e3
             rows.append((float(np.median(col)), name, float(col.min()), float(col.max())))
-    print(f"# job {jb} (DP step {jb + 1}, layer {jb}) of a search: model {cfg.name}, ctx {C}, M {M}, T {T}; us after the job's first stamp")
+    print(f"# job {jb} (DP step {jb + 2}, layer {jb + 1}) of a search: model {cfg.name}, ctx {C}, M {M}, T {T}; us after the job's first stamp")
     for med, name, lo, hi in sorted(rows):
         print(f"{name:28s} min {lo:8.2f}  median {med:8.2f}  max {hi:8.2f}")
     starts = [s[:, j * TRACE_SLOTS][s[:, j * TRACE_SLOTS] > 0].min() for j in range(L) if (s[:, j * TRACE_SLOTS] > 0).any()]
