@@ -208,8 +208,7 @@ struct clasp_ctx {
   bool use_engine = false;
   int e_G = 0;              // CTAs of the cooperative grid (one per SM)
   int e_static_smem = 0;
-  const void* e_kernel[4] = {nullptr, nullptr, nullptr, nullptr};   // the layer kernel for this head dimension: plain, with step
-                                                                    // stamps; [2], [3]: the same with the tensor-core attention
+  const void* e_kernel[2 * clasp::pk::N_KINDS] = {};   // the layer kernel for this head dimension by kind, plain and with step stamps
   int e_split_lo[clasp::pk::N_SPLITS], e_split_units[clasp::pk::N_SPLITS], e_tile_idx[5], e_tiles_off = 0,
       e_kpi[5], e_use3d[5], e_wpages[5];
   int e_heights[8][clasp::pk::N_HEIGHTS];   // tile heights per matrix slot (wq wk wv wo gate up down head)
@@ -808,11 +807,17 @@ int engine_setup(clasp_ctx* ctx) {
   const int d = c.d_model, qd = c.n_q_heads * c.head_dim, kvd = c.n_kv_heads * c.head_dim;
   if (d % 8 || c.d_ffn % 8 || c.vocab % 8) return CLASP_OK;
   // the instantiations for this model's head dimension, without and with step stamps
-  ctx->e_kernel[0] = c.head_dim == 128 ? (const void*)pk::engine_kernel<false, 128, false> : (const void*)pk::engine_kernel<false, 64, false>;
-  ctx->e_kernel[1] = c.head_dim == 128 ? (const void*)pk::engine_kernel<true, 128, false> : (const void*)pk::engine_kernel<true, 64, false>;
-  ctx->e_kernel[2] = c.head_dim == 128 ? (const void*)pk::engine_kernel<false, 128, true> : nullptr;
-  ctx->e_kernel[3] = c.head_dim == 128 ? (const void*)pk::engine_kernel<true, 128, true> : nullptr;
-  const int n_kern = c.head_dim == 128 ? 4 : 2;
+  const bool h128 = c.head_dim == 128;
+#define CLASP_KERNELS(k)                                                                                                       \
+  ctx->e_kernel[2 * (k)] = h128 ? (const void*)pk::engine_kernel<false, 128, k> : (const void*)pk::engine_kernel<false, 64, k>; \
+  ctx->e_kernel[2 * (k) + 1] = h128 ? (const void*)pk::engine_kernel<true, 128, k> : (const void*)pk::engine_kernel<true, 64, k>
+  CLASP_KERNELS(pk::K_SEARCH);
+  CLASP_KERNELS(pk::K_FORWARD);
+  CLASP_KERNELS(pk::K_MANY);
+#undef CLASP_KERNELS
+  ctx->e_kernel[2 * pk::K_TC] = h128 ? (const void*)pk::engine_kernel<false, 128, pk::K_TC> : nullptr;
+  ctx->e_kernel[2 * pk::K_TC + 1] = h128 ? (const void*)pk::engine_kernel<true, 128, pk::K_TC> : nullptr;
+  const int n_kern = h128 ? 2 * pk::N_KINDS : 2 * pk::K_TC;
   ctx->e_static_smem = 0;
   for (int k = 0; k < n_kern; ++k) {  // one shared-memory budget for both
     cudaFuncAttributes fa;
@@ -997,7 +1002,9 @@ int engine_launch(clasp_ctx* ctx, int Rmax, int head_off, clasp::SetupArgs setup
     att_tc = att_tc && J.type != pk::JOB_HEAD && !(J.type == pk::JOB_LAYER && (J.uniform || !J.dp));
   // (row, query head) pairs of a kv head: up to 64 of them fit an M = 64 accumulator, which leaves the ring 24 KB more
   const int att_rows = att_pairs <= 64 ? 64 : pk::TC_ROWS;
-  const int scratch_bytes = !att_tc ? pk::SCRATCH_BYTES : (att_rows == 64 ? pk::SCRATCH_TC64_BYTES : pk::SCRATCH_TC_BYTES);
+  const int n_slice = ctx->e_wpages[pk::G_DOWN] * 8;   // features of the largest o / down slice
+  const int scratch_bytes = std::max(pk::scratch_bytes(BN, n_slice),
+                                     !att_tc ? 0 : (att_rows == 64 ? pk::SCRATCH_TC64_BYTES : pk::SCRATCH_TC_BYTES));
   const int ring_pages = (optin - ctx->e_static_smem - 1024 - scratch_bytes) / pk::PAGE;
   // an item (gate + up rows and the operand tiles of kpi chunks) must fit the ring twice over
   const int b_pages = BN * pk::BK * 2 / pk::PAGE;
@@ -1088,9 +1095,14 @@ int engine_launch(clasp_ctx* ctx, int Rmax, int head_off, clasp::SetupArgs setup
   // The forward passes cut the cache into runs of a length fixed by the context capacity, so that a
   // position's attention is summed in the same order whichever call computes it (verification and
   // one-token decoding must agree bit for bit).  The search only has to agree with itself: it cuts
-  // the keys it sees into at most 32 runs, which spreads a short context over many more CTAs.
-  if (search_ctx >= 0) P.c.run_len = pk::ATT_KEYS * ((search_ctx + pk::ATT_KEYS * 32 - 1) / (pk::ATT_KEYS * 32) > 0
-                                                       ? (search_ctx + pk::ATT_KEYS * 32 - 1) / (pk::ATT_KEYS * 32) : 1);
+  // the keys it sees by the context and the head counts alone (not by its rows: a row's sums must not
+  // depend on how many share the launch) into so many runs that a kv head's runs and its own-key chunk are
+  // one chunk per CTA, and at most 16 where more do not fit (one trip of the merge).
+  if (search_ctx >= 0) {
+    const int per_head = std::max(1, ctx->e_G / c.n_kv_heads - 1);
+    const int runs = per_head >= 32 ? 32 : std::min(per_head, 16);
+    P.c.run_len = pk::ATT_KEYS * std::max(1, (search_ctx + pk::ATT_KEYS * runs - 1) / (pk::ATT_KEYS * runs));
+  }
   if (att_tc) {
     // run length: whole 64-key tiles, at most 32 runs; the cut that needs the fewest tile steps when the
     // (kv head, run, pair block) items are dealt out to the CTAs (one more step per round for its set-up)
@@ -1106,13 +1118,13 @@ int engine_launch(clasp_ctx* ctx, int Rmax, int head_off, clasp::SetupArgs setup
     }
     P.c.run_len = best_len;
   }
-  P.c.BN = BN; P.c.ring_pages = ring_pages; P.c.att_tc = att_tc ? 1 : 0; P.c.att_rows = att_rows;
+  P.c.BN = BN; P.c.ring_pages = ring_pages; P.c.stage_bytes = BN * n_slice * 4; P.c.att_tc = att_tc ? 1 : 0; P.c.att_rows = att_rows;
 
   for (int s = 0; s < pk::N_SPLITS; ++s) { P.c.split_lo[s] = ctx->e_split_lo[s]; P.c.split_units[s] = ctx->e_split_units[s]; }
   for (int k = 0; k < 5; ++k) { P.c.tile_idx[k] = ctx->e_tile_idx[k]; P.c.kpi[k] = kpi[k]; P.c.use3d[k] = use3d[k]; }
   P.c.tiles_off = ctx->e_tiles_off; P.c.map3d_off = (int)(((size_t)c.L * 7 + 1) * pk::N_HEIGHTS);
   P.b.xn_a = (bf16*)ws.xn; P.b.xn_m = (bf16*)ws.xn_m; P.b.attn = (bf16*)ws.attn; P.b.act = (bf16*)ws.act;
-  P.b.qkv = ws.qkv; P.b.x1 = ws.x1; P.b.Gbuf = ws.G; P.b.att_acc = ws.e_att_acc; P.b.att_ml = ws.e_att_ml;
+  P.b.qkv = ws.qkv; P.b.x1 = ws.x1; P.b.att_acc = ws.e_att_acc; P.b.att_ml = ws.e_att_ml;
   P.b.ss_a = ws.ss_a; P.b.ss_m = ws.ss_m; P.b.cosacc = ws.cosacc; P.b.head_best = ws.head_best; P.b.flags = ws.flags;
   P.b.rope = ws.rope;
   P.jobs = ws.jobs; P.n_jobs = (int)ctx->e_jobs.size(); P.wmaps = ws.wmaps; P.kvmaps = ws.kvmaps; P.tabs = ws.tabs; P.ctl = ws.ctl;
@@ -1133,7 +1145,10 @@ int engine_launch(clasp_ctx* ctx, int Rmax, int head_off, clasp::SetupArgs setup
   void* args[] = {(void*)&bm->second[0], (void*)&bm->second[1], (void*)&bm->second[2], (void*)&bm->second[3],
                   (void*)&hm->second[0], (void*)&bm->second[4], (void*)&bm->second[5], (void*)&bm->second[6],
                   (void*)&bm->second[7], (void*)&hm->second[1], (void*)&bm->second[8], (void*)&bm->second[9], (void*)&P};
-  const void* kern = ctx->e_kernel[(att_tc ? 2 : 0) + (ctx->e_trace ? 1 : 0)];
+  // (pairs of more than one block: their attention carries q from chunk to chunk, 20 us of a 150 us layer at 192 pairs over 2048
+  // positions; of one block, and the epilogues of a forward's few rows: figures at attention_one and epilogue_fwd)
+  const int kind = att_tc ? pk::K_TC : (att_pairs > 128 ? pk::K_MANY : (search_ctx >= 0 ? pk::K_SEARCH : pk::K_FORWARD));
+  const void* kern = ctx->e_kernel[2 * kind + (ctx->e_trace ? 1 : 0)];
   cudaError_t err = cudaLaunchCooperativeKernel(kern, dim3(ctx->e_G), dim3(pk::THREADS),
                                                 args, dyn, ctx->stream);
   if (ctx->profiling) {

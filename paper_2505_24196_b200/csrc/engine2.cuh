@@ -62,13 +62,17 @@ constexpr int TC_ROWS = 128;                  // (row, query head) pairs of one 
 constexpr int SCRATCH_TC64_BYTES = 57 * 1024; // the same with 64 rows per item: q tile 16 KB, P tile 8 KB
 constexpr int SCRATCH_TC_BYTES = 81 * 1024;   // q tile 32 KB, K, V and P tiles 16 KB each (1024-aligned), 1 KB of per-row words
 constexpr int MAX_ROWS = 128;         // rows one launch may push through a layer
-// Rows (accumulator columns) a worker group finishes per pass; the two groups of four warps take alternate
-// blocks.  4 or 8: with 4 the unrolled per-row code is half as long and 5 to 8 rows already keep both groups
-// busy (measured against 8: 8B search -0.5 %, forward passes -1.7 %, 8192-key contexts -3 %; launches with
-// many rows make more passes: 70B search with 32 rows +0.6 %, 128-row prefill +3 %).
-constexpr int RB = 4;
+constexpr int RB = 4;                 // rows a worker group finishes per pass of epilogue_fwd
+constexpr int PF = 4;                 // passes of the workers over a CTA's rows whose loads are in flight together
 constexpr int N_HEIGHTS = 4;          // distinct tile heights (TMA box heights) per weight matrix
 constexpr int MAX_CTAS = 192;
+// worker scratch of a launch of BN accumulator rows whose o / down slices have at most n features: the slice of every row
+// and four floats per row; never less than the attention tiles
+constexpr int EPI_TAB_BYTES = MAX_ROWS * 16;
+inline int scratch_bytes(int BN, int n) {
+  const int e = BN * n * 4 + EPI_TAB_BYTES;
+  return (e > SCRATCH_BYTES ? e + 1023 : SCRATCH_BYTES) & ~127;
+}
 
 enum { JOB_LAYER = 0, JOB_HEAD = 1, JOB_SELECT = 2 };
 enum { G_QKV = 0, G_O = 1, G_GU = 2, G_DOWN = 3, G_HEAD = 4 };
@@ -104,6 +108,7 @@ struct Cfg {
   int run_len, chunk_cap;
   int BN;              // activation rows padded to a multiple of 16 (MMA N)
   int ring_pages;
+  int stage_bytes;     // worker scratch taken by the slices of the launch's rows in an epilogue (the per-row floats follow)
   int att_rows;        // tensor-core attention: (row, query head) pairs per item, 64 or 128
   int att_tc;          // 1: search jobs run the attention over their cache keys on tcgen05 (kernel instantiation with
                        // TC set; the launch carries SCRATCH_TC_BYTES of worker scratch instead of SCRATCH_BYTES)
@@ -125,7 +130,6 @@ struct Bufs {
   bf16* act;       // [rows, dffn] operand of the down product
   float* qkv;      // [rows, qd + 2 kvd] projections (norm factor applied, not rotated)
   float* x1;       // [rows, d]    residual stream after attention
-  float* Gbuf;     // [rows, d]    layer outputs of the candidate states (Eq. 2)
   uint2* att_acc;  // [rows*nq, chunk_cap, hd / 2] partial attention outputs: (two bf16 values, tag) per 8 bytes
   uint4* att_ml;   // [rows*nq, chunk_cap] (running maximum, tag, sum, tag)
   long long* ss_a; // [jobs, Rcap] row sums of squares of the operand of job j's first product (attention
@@ -356,23 +360,25 @@ struct Shared {
   volatile int abort;
   uint32_t wait_fast, wait_slow;   // the launch's wait limits
   volatile int a_issued;    // ring items whose weight loads have been issued (warp 0 -> warp 1)
+  int b_seen;               // products whose operand warp 1 has seen complete (warp 1 -> workers)
   int flag;                 // broadcast of a one-thread decision to the workers
   float rs[MAX_ROWS];       // per-row norm factors of the current product
   float rs_next[MAX_ROWS];  // Eq. 2 step: norm factors of the rows it hands to the next layer
-  int choice[MAX_ROWS + 2];   // Eq. 2 decision per state (1: the layer output was taken)
-  int choice_row[MAX_ROWS + 16];  // the same per candidate row
+  int choice_row[MAX_ROWS + 16];  // Eq. 2 decision per candidate row (1: the layer output was taken)
   int foot[NB];             // warp 0: ring pages each item in flight gives back when it retires
   alignas(16) int job_words[(sizeof(Job) + 3) / 4];  // the workers' copy of the current job descriptor (read back as a
                                                      // Job: its pointer fields need 8-byte alignment)
 };
-// The workers' scratch area holds either the attention K/V tiles or, during epilogues and the
-// Eq. 2 step, the cross-warp reduction tables below (the two uses never overlap in time).
-constexpr int RED_ROWS = MAX_ROWS + 16;
-struct RedTables {
-  float red[4][RED_ROWS][5];   // [lane quarter][row][value]: per-row sums of one warp
-  double cosv[RED_ROWS][5];
+// The workers' scratch area holds the attention's K/V tiles or, in an epilogue and the Eq. 2 step, the accumulators of the
+// CTA's slice by row ([row][feature], Cfg::stage_bytes) and then four floats per row, or, in the LM head's epilogue, these
+// tables (the uses never overlap in time).
+struct HeadTables {
+  float red[4][MAX_ROWS][3];   // [lane quarter][row]: best logit, its index, sum of exp
 };
-static_assert(sizeof(RedTables) <= SCRATCH_BYTES, "reduction tables must fit the scratch area");
+struct RowTables {   // (epilogue_fwd)
+  float red[4][MAX_ROWS][3];   // [lane quarter][row][value]: per-row sums of one warp
+};
+static_assert(sizeof(HeadTables) <= SCRATCH_BYTES && sizeof(RowTables) <= SCRATCH_BYTES, "tables must fit the scratch area");
 
 constexpr uint32_t POLL_NS = 100;      // pause between two polls of a flag or counter in global memory: the line is polled
                                        // by every CTA while the last ones still add to it (no pause: +0.7 % on the 8B search)
@@ -395,8 +401,10 @@ __device__ __forceinline__ bool aborted(Ctl* ctl, Shared* sh) {
 __device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, Ctl* ctl, Shared* sh) {
   const uint32_t b = tc::smem_u32(bar);
   const uint32_t n_fast = sh->wait_fast, n_slow = sh->wait_slow;
+#pragma unroll 1
   for (uint32_t it = 0; it < n_fast; ++it)
     if (tc::mbar_test(b, parity)) return true;
+#pragma unroll 1
   for (uint32_t it = 0; it < n_slow; ++it) {
     if (tc::mbar_test(b, parity)) return true;
     if (aborted(ctl, sh)) return false;
@@ -409,6 +417,7 @@ __device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, Ctl* ct
 // Bounded wait until flag >= epoch.
 __device__ __forceinline__ bool wait_flag(const int* flag, int epoch, Ctl* ctl, Shared* sh) {
   const uint32_t n = 2u * sh->wait_slow;
+#pragma unroll 1
   for (uint32_t it = 0; it < n; ++it) {
     if (ld_acquire_i32(flag) >= epoch) return true;
     __nanosleep(POLL_NS);
@@ -459,7 +468,7 @@ struct Phase {   // one product of one job, as seen by this CTA
     tile0 = __ldg(ti);
     n_tiles = __ldg(ti + 1) - tile0;
     map_base = kind_map_base(c, kind, J.layer);
-    g0 = (int)(((long long)blockIdx.x * n_groups) / c.G);
+    g0 = ((int)blockIdx.x * n_groups) / c.G;
   }
   __device__ __forceinline__ int group_at(int gi) const {
     const int g = g0 + gi;
@@ -610,9 +619,12 @@ __device__ void producer_b(const Params& p, Shared* sh, uint32_t ring_base, cons
   RingPos rp{0, 0};
   const int b_pages = (c.BN * BK * 2) / PAGE;
   const uint32_t b_bytes = (uint32_t)c.BN * BK * 2;
+  int n_seen = 0;
+#pragma unroll 1
   for (int jb = 0; jb < p.n_jobs; ++jb) {
     const Job& J = p.jobs[jb];
     const int nph = n_gemm_phases(J);
+#pragma unroll 1
     for (int ph = 0; ph < nph; ++ph) {
       Phase P;
       P.init(p, J, ph);
@@ -629,15 +641,19 @@ __device__ void producer_b(const Params& p, Shared* sh, uint32_t ring_base, cons
         bool ok = true;
         if (lane == 0) ok = wait_count(p, fkind, tgt, sh);
         if (!__all_sync(0xffffffffu, ok)) return;
+        ++n_seen;
+        if (lane == 0) asm volatile("st.release.cta.shared::cta.s32 [%0], %1;" ::"r"(tc::smem_u32(&sh->b_seen)), "r"(n_seen) : "memory");
         if (lane == 0 && P.kind < 3) issuer_mark<TR>(p, jb, T_B_READY + P.kind);
       }
       fence_proxy_async();  // the producers' ordinary stores before this warp's TMA reads
       const bool d3 = c.use3d[P.kind] != 0;
+#pragma unroll 1
       for (int t = 0; t < P.n_tiles; ++t) {
         const TileDesc td = tiles[P.tile0 + t];
         const int w_pages = (P.dual + 1) * (td.n_rows >> 3);
         const int pages = P.kpi * (w_pages + P.bmul * b_pages);
         const uint32_t pb_bytes = (uint32_t)P.bmul * b_bytes;   // operand tile of one chunk
+#pragma unroll 1
         for (int gi = 0; gi < P.n_groups; ++gi) {
           int fp;
           const uint32_t it = rp.item;
@@ -645,6 +661,7 @@ __device__ void producer_b(const Params& p, Shared* sh, uint32_t ring_base, cons
           // the weight producer has made room for this item
           bool ok = false;
           const uint32_t n_fast = sh->wait_fast, n_slow = sh->wait_slow;
+#pragma unroll 1
           for (uint32_t w = 0; w < n_slow; ++w) {
             if ((uint32_t)sh->a_issued > it) { ok = true; break; }
             if (w > n_fast) {
@@ -685,12 +702,15 @@ __device__ void mma_issuer(const Params& p, Shared* sh, uint32_t ring_base, uint
   const int b_pages = (c.BN * BK * 2) / PAGE;
   uint32_t n_acc = 0;
   const uint32_t el = elect_one();
+#pragma unroll 1
   for (int jb = 0; jb < p.n_jobs; ++jb) {
     const Job& J = p.jobs[jb];
     const int nph = n_gemm_phases(J);
+#pragma unroll 1
     for (int ph = 0; ph < nph; ++ph) {
       Phase P;
       P.init(p, J, ph);
+#pragma unroll 1
       for (int t = 0; t < P.n_tiles; ++t) {
         const TileDesc td = tiles[P.tile0 + t];
         const int a_pages = td.n_rows >> 3;
@@ -708,6 +728,7 @@ __device__ void mma_issuer(const Params& p, Shared* sh, uint32_t ring_base, uint
         const uint64_t w_lo = (uint64_t)(w_pages * (PAGE / 16));               // weights of one chunk
         const uint64_t x_lo = (uint64_t)(P.bmul * b_pages * (PAGE / 16));      // operand tile of one chunk
         const uint64_t x0_lo = (uint64_t)P.kpi * w_lo;                         // first weight chunk -> first operand tile
+#pragma unroll 1
         for (int gi = 0; gi < P.n_groups; ++gi) {
           int fp;
           const uint32_t it = rp.item;
@@ -754,16 +775,20 @@ __device__ void mma_issuer(const Params& p, Shared* sh, uint32_t ring_base, uint
 // ------------------------------------------------------------------ worker steps
 // TR: the step stamps are compiled in; HD: the model's head dimension (64 or 128).  The kernel is
 // sensitive to its code size, so an instantiation carries neither stamps it does not take nor the
-// attention code of the other head dimension; TC: the instantiation for searches over long contexts (tensor-core
-// attention over the cache keys, Eq. 2 write-back dealt to all threads); it is launched for nothing else.
-template <bool TR, int HD, bool TC>
+// attention code of the other head dimension.  KIND: what it is launched for -- searches whose (row, query head) pairs of a kv
+// head are one block of 128 at most, other launches of such few pairs, launches of more pairs, searches over long contexts
+// (tensor-core attention over the cache keys).
+enum { K_SEARCH = 0, K_FORWARD = 1, K_MANY = 2, K_TC = 3, N_KINDS = 4 };
+template <bool TR, int HD, int KIND>
 struct Worker {
+  static constexpr bool TC = KIND == K_TC, MR = KIND == K_MANY, FW = KIND == K_FORWARD;
   const Params& p;
   Shared* sh;
   uint8_t* scratch;
   uint32_t tmem_base;
   int wtid, ww, lane;
   uint32_t n_acc;
+  int n_prod;               // products of this CTA so far
   int n_mark;
   uint32_t att_phase = 0;   // parity of att_bar's next completion
   uint32_t att_kph = 0, att_vph = 0;   // the same for the K / V tile barriers (worker warp 4)
@@ -810,7 +835,6 @@ struct Worker {
     return fl < n ? fl : -1;
   }
   __device__ __forceinline__ const int* split_lo(int split) const { return p.tabs + p.c.split_lo[split]; }
-  __device__ __forceinline__ RedTables* tables() const { return reinterpret_cast<RedTables*>(scratch); }
 
   // fixed-point scale of the sums of squares (2^24: sums up to 5e11, resolution 6e-8)
   static constexpr double SS_FIX = 16777216.0;
@@ -856,6 +880,70 @@ struct Worker {
     for (int i = 0; i < RB; ++i) v[i] = __uint_as_float(r[i]);
   }
 
+  // eight accumulator columns of this thread's lane (the caller waits: tmem_wait)
+  __device__ __forceinline__ static void tmem_ld8(uint32_t taddr, float (&v)[8]) {
+    uint32_t r[8];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+  }
+  // (the values pass through the wait, so that nothing reads them before it)
+  __device__ __forceinline__ static void tmem_wait(float (&v)[8]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7])::"memory");
+  }
+
+  // A CTA's slice of n features (a multiple of 8, at most 128) over the rows, dealt to the workers by row: the four-feature
+  // pieces of a row sit in 2^lq neighbouring lanes (so that a row's sums are shuffles inside the group), a thread keeps
+  // its piece from pass to pass.  All threads of a warp make the same passes.
+  struct Slice {
+    int lq, q, r0, step;
+    bool on;
+    __device__ __forceinline__ Slice(int n, int wtid) {
+      const int n4 = n >> 2;
+      lq = n4 > 1 ? 32 - __clz(n4 - 1) : 0;
+      q = wtid & ((1 << lq) - 1);
+      r0 = wtid >> lq;
+      step = WORKERS >> lq;
+      on = q < n4;
+    }
+    __device__ __forceinline__ int passes(int rows) const { return (rows + step - 1) >> (8 - lq); }
+  };
+  static_assert(WORKERS == 256, "a slice's passes are counted with shifts");
+  template <int N>
+  __device__ __forceinline__ static void group_sum(float (&v)[N], int lq) {
+#pragma unroll 1
+    for (int o = 1; o < (1 << lq); o <<= 1) {
+#pragma unroll
+      for (int i = 0; i < N; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
+    }
+  }
+  // Sum of squares of a row's n features from the four that each thread of the group holds, in the order of epilogue_fwd (a
+  // row is the same bits in either): inside the lane quarters of the accumulator (16 features, 32 past 64) by lane distances
+  // 2, 1, 4, 8, 16, then the quarters one by one.
+  __device__ __forceinline__ static float row_square(const float4& y, int n, int lq) {
+    float t = __fadd_rn(__fadd_rn(__fmul_rn(y.x, y.x), __fmul_rn(y.z, y.z)), __fadd_rn(__fmul_rn(y.y, y.y), __fmul_rn(y.w, y.w)));
+    const int qq = n <= 64 ? 2 : 3;       // log2 of a quarter's threads
+#pragma unroll 1
+    for (int o = 1; o < (1 << (lq < qq ? lq : qq)); o <<= 1) t = __fadd_rn(t, __shfl_xor_sync(0xffffffffu, t, o));
+    if (lq <= qq) return t;
+    const int first = (int)(threadIdx.x & 31u) & ~((1 << lq) - 1);
+    float sum = __shfl_sync(0xffffffffu, t, first);
+#pragma unroll 1
+    for (int k = 1; k < (1 << (lq - qq)); ++k) sum = __fadd_rn(sum, __shfl_sync(0xffffffffu, t, first + (k << qq)));
+    return sum;
+  }
+  __device__ __forceinline__ static float dot4(const float4& a, const float4& b) {
+    return (a.x * b.x + a.y * b.y) + (a.z * b.z + a.w * b.w);
+  }
+  __device__ __forceinline__ static void st_bf16x4(bf16* dst, const float4& y, const float4& w) {
+    *reinterpret_cast<uint2*>(dst) = pack4(y.x * w.x, y.y * w.y, y.z * w.z, y.w * w.w);
+  }
+  __device__ __forceinline__ static float4 ld4(const float* src) { return __ldcg(reinterpret_cast<const float4*>(src)); }
+  __device__ __forceinline__ float* stage() const { return reinterpret_cast<float*>(scratch); }
+
   // per-row factors rsqrt(mean(x^2) + eps) from the accumulated sums of squares
   __device__ void row_scales(const long long* ss, int R, int row_off) {
     const Cfg& c = p.c;
@@ -887,57 +975,272 @@ struct Worker {
     publish(F_PREP, epoch);
   }
 
-  // ---- epilogue of one accumulator: tile td of product P.kind.
-  // Thread (quarter q, lane) owns feature td.f0 + 32 q + lane; the two warps of a quarter take
-  // alternating blocks of RB rows (accumulator columns).  Per-row sums over the CTA's features
-  // (sums of squares, cosine partials, arg-max) go through RedTables: one entry per (quarter, row).
-  // For the down product of an Eq. 2 job the thread's layer outputs (keep_y) and skip candidates
-  // (keep_s) of its first block of RB rows stay in registers for dp_step.
-  __device__ bool epilogue(const Job& J, int jb, const Phase& P, const TileDesc& td, int tile_no, float (&keep_y)[RB],
-                           float (&keep_s)[RB]) {
+  // The product's next accumulator is complete: one thread polls the barrier, the others sleep in the hardware barrier behind it.
+  __device__ __forceinline__ bool acc_wait(uint32_t buf) {
+    bool ok = true;
+    if (wtid == 0) ok = wait_bar(&sh->acc_full[buf], (n_acc >> 1) & 1u, p.ctl, sh);
+    ok = worker_and(ok);
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    return ok;
+  }
+  // all workers have read the accumulator: the issuer may overwrite it
+  __device__ __forceinline__ void acc_free(uint32_t buf) {
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    worker_sync();
+    if (wtid == 0) mbar_arrive(tc::smem_u32(&sh->acc_empty[buf]));
+    ++n_acc;
+  }
+  // The product's operand is complete, so every CTA's sums of squares are too: its rows' norm factors are made while it is
+  // being multiplied (behind the accumulator they would cost a trip to L2).  Warp 1 has polled the counter already.
+  __device__ bool row_scales_early(const long long* ss, int R, int row_off) {
+    bool ok = true;
+    if (wtid == 0) {
+      ok = false;
+      const uint32_t n = sh->wait_slow;
+#pragma unroll 1
+      for (uint32_t it = 0; it < n; ++it) {
+        int v;
+        asm volatile("ld.acquire.cta.shared::cta.s32 %0, [%1];" : "=r"(v) : "r"(tc::smem_u32(&sh->b_seen)) : "memory");
+        if (v > n_prod) { ok = true; break; }
+        if (aborted(p.ctl, sh)) break;
+        __nanosleep(20);
+      }
+      if (!ok && !aborted(p.ctl, sh)) raise_abort(p.ctl, sh, true);
+    }
+    if (!worker_and(ok)) return false;
+    row_scales(ss, R, row_off);
+    return true;
+  }
+
+  // ---- epilogue of a q/k/v or gate/up accumulator: thread (lane quarter, lane) owns a feature, the two warps of a quarter
+  // take alternate blocks of eight rows (accumulator columns).
+  __device__ bool epilogue_features(const Job& J, int jb, const Phase& P, const TileDesc& td, int tile_no) {
     const Cfg& c = p.c;
-    RedTables* T = tables();
     const int quarter = ww & 3, group = ww >> 2;
     const int fl = feat_local(td.n_rows, quarter, lane);
     const bool fv = fl >= 0;
     const int f = td.f0 + fl;
-    const bool dpd = P.kind == G_DOWN && J.dp;
-    const int rows_all = J.R + ((dpd && J.diag) ? J.T : 0);   // Eq. 2: plus the rows of the diagonal state
-    const int ncb = (J.R + RB - 1) / RB;
-    const bool resid = P.kind == G_O || P.kind == G_DOWN;
-    const RowDiv rd(J.T);
-    // Eq. 2: objective row and skip candidate of every row of the first block, fetched early
-    float xi[RB];
-    if (dpd) {
+    const bool from_step = P.kind == G_QKV && (J.src_flag == F_SELECT || J.dual_src);
+    if (tile_no == 0 && !from_step) {
+      if (!row_scales_early((P.kind == G_GU ? p.b.ss_m : p.b.ss_a) + (long long)jb * c.Rcap, J.R, 0)) return false;
+    }
+    if (tile_no == 0 && from_step) {   // the rows come from an Eq. 2 step: it left their factors in shared memory
+      for (int r = wtid; r < J.R; r += WORKERS) sh->rs[r] = sh->rs_next[r + J.in_shift];
+    }
+    const uint32_t buf = n_acc & 1u;
+    if (!acc_wait(buf)) return false;
+    if (tile_no == 0) mark(T_ACC + P.kind);
+    const uint32_t t_lane = tmem_base + buf * 256u + ((uint32_t)(quarter * 32) << 16);
+    const bool two = P.dual || P.bmul == 2;
+    const int r_end = __any_sync(0xffffffffu, fv) ? J.R : 0;   // (a warp without a feature has nothing to do)
+#pragma unroll 1
+    for (int c0 = group * 8; c0 < r_end; c0 += 16) {
+      float v[8], u[8];
+      tmem_ld8(t_lane + (uint32_t)c0, v);
+      if (two) {
+        tmem_ld8(t_lane + (uint32_t)(c.BN + c0), u);
+        tmem_wait(u);
+      }
+      tmem_wait(v);
+      if (P.kind == G_QKV) {
+        float* dst = p.b.qkv + (long long)c0 * (c.qd + 2 * c.kvd) + f;
 #pragma unroll
-      for (int k = 0; k < RB; ++k) {
-        const int r = group * RB + k;
-        xi[k] = 0.f;
-        keep_s[k] = 0.f;
-        keep_y[k] = 0.f;
-        if (fv && r < rows_all) {
-          xi[k] = __ldg(J.x_i + rd.mod(r) * J.x_tok_stride + f);
-          keep_s[k] = __ldcg(skip_row(J, r) + f);
+        for (int k = 0; k < 8; ++k) {
+          if (fv && c0 + k < J.R) {
+            // (both candidates of every state went through the product, v: layer output, u: skip candidate: the one the
+            // Eq. 2 step chose counts)
+            const float x = P.bmul == 2 && !sh->choice_row[c0 + k + J.in_shift] ? u[k] : v[k];
+            __stcg(dst, x * sh->rs[c0 + k]);
+          }
+          dst += c.qd + 2 * c.kvd;
+        }
+      } else {
+        bf16* dst = p.b.act + (long long)c0 * c.dffn + f;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          if (fv && c0 + k < J.R) {
+            const float rs = sh->rs[c0 + k];
+            *dst = __float2bfloat16_rn(silu_f(rs * v[k]) * (rs * u[k]));
+          }
+          dst += c.dffn;
         }
       }
-      if (J.defer && fv) {   // the skip candidates' rows of the next layer's operand
-        const float wq = __ldg(J.norm_next + f);
+    }
+    acc_free(buf);
+    return true;
+  }
+
+  // ---- epilogue of the LM head: per row the tile's best logit (lowest index on ties) and sum of exp
+  __device__ bool epilogue_head(const Job& J, int jb, const TileDesc& td, int tile_no) {
+    const Cfg& c = p.c;
+    HeadTables* T = reinterpret_cast<HeadTables*>(scratch);
+    const int quarter = ww & 3, group = ww >> 2;
+    const int fl = feat_local(td.n_rows, quarter, lane);
+    const bool fv = fl >= 0;
+    const int f = td.f0 + fl;
+    const uint32_t buf = n_acc & 1u;
+    // (a head over the last rows of the job before it: their sums of squares start at row_off)
+    if (tile_no == 0 && !row_scales_early(p.b.ss_a + (long long)jb * c.Rcap, J.R, J.row_off)) return false;
+    if (!acc_wait(buf)) return false;
+    const uint32_t t_lane = tmem_base + buf * 256u + ((uint32_t)(quarter * 32) << 16);
+#pragma unroll 1
+    for (int r = group; r < J.R; r += 2) {
+      uint32_t raw;
+      asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(raw) : "r"(t_lane + (uint32_t)r));
+      asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(raw)::"memory");
+      const float mine = fv ? __uint_as_float(raw) * sh->rs[r] : -INFINITY;
+      if (J.logits_out && fv) __stcg(J.logits_out + (long long)r * c.vocab + f, mine);
+      float best = mine;
+      int bi = fv ? f : 0x7fffffff;
 #pragma unroll
-        for (int k = 0; k < RB; ++k) {
-          const int r = group * RB + k;
-          if (r < rows_all) p.b.xn_a[(long long)(c.BN + r) * c.d + f] = __float2bfloat16_rn(keep_s[k] * wq);
+      for (int o = 16; o > 0; o >>= 1) {
+        const float ov = __shfl_xor_sync(0xffffffffu, best, o);
+        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+        if (ov > best || (ov == best && oi < bi)) { best = ov; bi = oi; }
+      }
+      const float se = warp_sum(fv ? __expf(mine - best) : 0.f);
+      if (lane == 0) {
+        T->red[quarter][r][0] = best;
+        T->red[quarter][r][1] = __int_as_float(bi);
+        T->red[quarter][r][2] = se;
+      }
+    }
+    acc_free(buf);
+    for (int r = wtid; r < J.R; r += WORKERS) {
+      float best = -INFINITY, se = 0.f;
+      int bi = 0x7fffffff;
+      for (int q4 = 0; q4 < 4; ++q4) {
+        const float ov = T->red[q4][r][0];
+        const int oi = __float_as_int(T->red[q4][r][1]);
+        if (ov > best || (ov == best && oi < bi)) { best = ov; bi = oi; }
+      }
+      for (int q4 = 0; q4 < 4; ++q4) {
+        const float ov = T->red[q4][r][0];
+        if (ov != -INFINITY) se += T->red[q4][r][2] * __expf(ov - best);
+      }
+      float4* dst = p.b.head_best + (long long)blockIdx.x * MAX_ROWS + r;
+      if (tile_no > 0) {
+        const float4 o = *dst;
+        const int oi = __float_as_int(o.y);
+        const float nb = fmaxf(o.x, best);
+        se = se * __expf(best - nb) + o.z * __expf(o.x - nb);
+        if (o.x > best || (o.x == best && oi < bi)) { best = o.x; bi = oi; }
+      }
+      *dst = make_float4(best, __int_as_float(bi), se, 0.f);
+    }
+    worker_sync();   // tables reused by the next tile
+    return true;
+  }
+
+  // ---- epilogue of an o or down accumulator (the CTA's slice of the d features): the accumulator goes to shared memory by
+  // row, then the slice is dealt to all workers by row (Slice): 16-byte accesses to the residual stream, sums over the
+  // slice without a table, and the residual rows of the first PF passes in flight while the product is multiplied.
+  // (A thread per feature used a quarter of the workers for a slice of 28 features and walked the rows one L2 trip after
+  // the other.)  An Eq. 2 job's layer outputs stay in the staged rows for dp_step.
+  __device__ bool epilogue_rows(const Job& J, int jb, int kind, const TileDesc& td, float4& keep_s) {
+    const Cfg& c = p.c;
+    const int n = td.n_rows;
+    const Slice sl(n, wtid);
+    const int f = td.f0 + 4 * sl.q;
+    const bool o_prod = kind == G_O, dpd = !o_prod && J.dp;
+    const float* res = (o_prod ? J.x_in : p.b.x1) + f;
+    const long long ldr = o_prod ? J.ldx : (long long)c.d;
+    const RowDiv rd(J.T);
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 rv[PF], xv[PF];
+    auto fetch = [&](int pass0) {
+#pragma unroll
+      for (int k = 0; k < PF; ++k) {
+        const int r = sl.r0 + (pass0 + k) * sl.step;
+        rv[k] = zero;
+        xv[k] = zero;
+        if (sl.on && r < J.R) {
+          rv[k] = ld4(res + r * ldr);
+          if (dpd) xv[k] = __ldg(reinterpret_cast<const float4*>(J.x_i + rd.mod(r) * J.x_tok_stride + f));
         }
-        for (int cb = group + 2; cb * RB < rows_all; cb += 2) {
+      }
+    };
+    fetch(0);
+    const float* nw = o_prod ? J.norm_mlp : ((!J.dp || J.defer) ? J.norm_next : nullptr);
+    float4 wn = zero;
+    if (sl.on && nw) wn = __ldg(reinterpret_cast<const float4*>(nw + f));
+    if (dpd) {
+      keep_s = zero;
+      if (sl.on && sl.r0 < J.R + (J.diag ? J.T : 0)) keep_s = ld4(skip_row(J, sl.r0) + f);
+    }
+    const uint32_t buf = n_acc & 1u;
+    if (!acc_wait(buf)) return false;
+    mark(T_ACC + kind);
+    {
+      const int quarter = ww & 3, fl = feat_local(n, quarter, lane);
+      const uint32_t t_lane = tmem_base + buf * 256u + ((uint32_t)(quarter * 32) << 16);
+      if (__any_sync(0xffffffffu, fl >= 0)) {
+#pragma unroll 1
+        for (int c0 = (ww >> 2) * 8; c0 < J.R; c0 += 16) {
+          float v[8];
+          tmem_ld8(t_lane + (uint32_t)c0, v);
+          tmem_wait(v);
+          float* dst = stage() + c0 * n + fl;
+          if (fl >= 0) {
 #pragma unroll
-          for (int k = 0; k < RB; ++k) {
-            const int r = cb * RB + k;
-            if (r < rows_all)
-              p.b.xn_a[(long long)(c.BN + r) * c.d + f] =
-                  __float2bfloat16_rn(__ldcg(skip_row(J, r) + f) * wq);
+            for (int k = 0; k < 8; ++k) dst[k * n] = v[k];   // (rows up to the padded count BN have a place)
           }
         }
       }
     }
+    acc_free(buf);
+    const int passes = sl.passes(J.R);
+    unsigned long long* acc =
+        reinterpret_cast<unsigned long long*>(p.b.cosacc) + (long long)jb * ((long long)(c.Rcap + MAX_ROWS) * 5);
+    long long* ss = o_prod ? p.b.ss_m + (long long)jb * c.Rcap : p.b.ss_a + (long long)(jb + 1) * c.Rcap;
+    float* out = o_prod ? p.b.x1 + f : (dpd ? nullptr : J.x_out + f);
+    const long long ldo = o_prod ? (long long)c.d : J.ldo;
+    bf16* xn = (o_prod ? p.b.xn_m : p.b.xn_a) + f;
+#pragma unroll 1
+    for (int pass0 = 0; pass0 < passes; pass0 += PF) {
+      if (pass0) fetch(pass0);
+#pragma unroll
+      for (int k = 0; k < PF; ++k) {
+        if (pass0 + k >= passes) break;
+        const int r = sl.r0 + (pass0 + k) * sl.step;
+        const bool ok = sl.on && r < J.R;
+        float4 y = zero;
+        if (ok) {
+          float4* at = reinterpret_cast<float4*>(stage() + r * n + 4 * sl.q);
+          y = *at;
+          y.x += rv[k].x; y.y += rv[k].y; y.z += rv[k].z; y.w += rv[k].w;
+          if (dpd) *at = y;
+          else __stcg(reinterpret_cast<float4*>(out + r * ldo), y);
+          if (nw) st_bf16x4(xn + (long long)r * c.d, y, wn);
+        }
+        if (dpd) {
+          // of the sums of Eq. 2 the two that involve the layer outputs (pre_sums has added the others)
+          float t[2] = {dot4(xv[k], y), dot4(y, y)};
+          group_sum(t, sl.lq);
+          if (ok && sl.q < 2) cos_add(acc + r * 5 + sl.q, sl.q ? t[1] : t[0]);
+        } else if (nw) {
+          // o product: MLP norm of this job; down product: the next job's first operand
+          const float t = row_square(y, n, sl.lq);
+          if (ok && sl.q == 0) ss_add(ss + r, t);
+        }
+      }
+    }
+    return true;
+  }
+
+  // ---- epilogue of one accumulator in the instantiation for forward passes of few rows: tile td of product P.kind.
+  // Thread (quarter q, lane) owns feature td.f0 + 32 q + lane; the two warps of a quarter take alternating blocks of RB rows
+  // (accumulator columns).  Per-row sums over the CTA's features go through RowTables: one entry per (quarter, row).  Of one
+  // to sixteen rows a layer takes 1.4 us less this way than through epilogue_rows; the sums are the same bits.
+  __device__ bool epilogue_fwd(const Job& J, int jb, const Phase& P, const TileDesc& td, int tile_no) {
+    const Cfg& c = p.c;
+    RowTables* T = reinterpret_cast<RowTables*>(scratch);
+    const int quarter = ww & 3, group = ww >> 2;
+    const int fl = feat_local(td.n_rows, quarter, lane);
+    const bool fv = fl >= 0;
+    const int f = td.f0 + fl;
+    const int ncb = (J.R + RB - 1) / RB;
+    const bool resid = P.kind == G_O || P.kind == G_DOWN;
     // residual rows of this thread's first two blocks are fetched before the accumulator is ready (a load
     // from L2 costs 1 - 2 us here; with twelve rows no block is left that would wait for one)
     float res[RB], res_n[RB];
@@ -954,8 +1257,11 @@ struct Worker {
     float wn = 0.f;
     if (fv) {
       if (P.kind == G_O) wn = __ldg(J.norm_mlp + f);
-      else if (P.kind == G_DOWN && (!J.dp || J.defer) && J.norm_next) wn = __ldg(J.norm_next + f);
+      else if (P.kind == G_DOWN && J.norm_next) wn = __ldg(J.norm_next + f);
     }
+    if ((P.kind == G_QKV || P.kind == G_GU || P.kind == G_HEAD) && tile_no == 0 &&
+        !row_scales_early((P.kind == G_GU ? p.b.ss_m : p.b.ss_a) + (long long)jb * c.Rcap, J.R, P.kind == G_HEAD ? J.row_off : 0))
+      return false;
     const uint32_t buf = n_acc & 1u;
     // one thread polls the barrier, the others sleep in the hardware barrier behind it
     bool ok = true;
@@ -964,28 +1270,11 @@ struct Worker {
     if (!ok) return false;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (tile_no == 0 && P.kind < 4) mark(T_ACC + P.kind);
-    if (P.kind == G_QKV && tile_no == 0 && (J.src_flag == F_SELECT || J.dual_src)) {
-      // the rows come from an Eq. 2 step: it left their factors in shared memory
-      for (int r = wtid; r < J.R; r += WORKERS) sh->rs[r] = sh->rs_next[r + J.in_shift];
-      worker_sync();
-    } else if ((P.kind == G_QKV || P.kind == G_GU || P.kind == G_HEAD) && tile_no == 0) {
-      // the reduction consumed every operand column, so every CTA's sums of squares are published
-      row_scales((P.kind == G_GU ? p.b.ss_m : p.b.ss_a) + (long long)jb * c.Rcap, J.R, P.kind == G_HEAD ? J.row_off : 0);
-    }
     const uint32_t t_lane = tmem_base + buf * 256u + ((uint32_t)(quarter * 32) << 16);
     for (int cb = group; cb < ncb; cb += 2) {
       float v[RB], u[RB];
       tmem_ld_rb(t_lane + (uint32_t)(cb * RB), v);
-      if (P.dual || P.bmul == 2) tmem_ld_rb(t_lane + (uint32_t)(c.BN + cb * RB), u);
-      if (P.bmul == 2) {
-        // both candidates of every state went through the product (v: layer output, u: skip candidate):
-        // keep the one the Eq. 2 step chose
-#pragma unroll
-        for (int k = 0; k < RB; ++k) {
-          const int r = cb * RB + k;
-          if (r < J.R && !sh->choice_row[r + J.in_shift]) v[k] = u[k];
-        }
-      }
+      if (P.dual) tmem_ld_rb(t_lane + (uint32_t)(c.BN + cb * RB), u);
       if (cb == group + 2) {
 #pragma unroll
         for (int k = 0; k < RB; ++k) res[k] = res_n[k];
@@ -1015,7 +1304,7 @@ struct Worker {
             __stcg(p.b.x1 + (long long)r * c.d + f, y);
             p.b.xn_m[(long long)r * c.d + f] = __float2bfloat16_rn(y * wn);
           }
-          sq[k] = y * y;
+          sq[k] = __fmul_rn(y, y);
         }
         const float tot = warp_reduce<RB>(sq, lane);
         if (lane < RB && cb * RB + lane < J.R) T->red[quarter][cb * RB + lane][0] = tot;
@@ -1030,29 +1319,6 @@ struct Worker {
             }
           }
         }
-      } else if (dpd) {
-        // layer outputs of the candidate states; per row the two sums of Eq. 2 that involve them
-        // (x.y and y.y; the sums over the skip candidates were added when those were written)
-        if (cb != group) {
-#pragma unroll
-          for (int k = 0; k < RB; ++k) {
-            const int r = cb * RB + k;
-            xi[k] = (fv && r < J.R) ? __ldg(J.x_i + rd.mod(r) * J.x_tok_stride + f) : 0.f;
-          }
-        }
-        float pr[2 * RB];
-#pragma unroll
-        for (int k = 0; k < RB; ++k) {
-          const int r = cb * RB + k;
-          const float y = (fv && r < J.R) ? res[k] + v[k] : 0.f;
-          if (fv && r < J.R && ncb > 2) __stcg(p.b.Gbuf + (long long)r * c.d + f, y);
-          if (J.defer && fv && r < J.R) p.b.xn_a[(long long)r * c.d + f] = __float2bfloat16_rn(y * wn);
-          if (cb == group) keep_y[k] = y;
-          pr[k] = xi[k] * y;
-          pr[RB + k] = y * y;
-        }
-        const float tot = warp_reduce<2 * RB>(pr, lane);
-        if (lane < 2 * RB && cb * RB + (lane & (RB - 1)) < J.R) T->red[quarter][cb * RB + (lane & (RB - 1))][lane / RB] = tot;
       } else if (P.kind == G_DOWN) {
         float sq[RB];
 #pragma unroll
@@ -1063,7 +1329,7 @@ struct Worker {
             __stcg(J.x_out + r * J.ldo + f, y);
             if (J.norm_next) p.b.xn_a[(long long)r * c.d + f] = __float2bfloat16_rn(y * wn);
           }
-          sq[k] = y * y;
+          sq[k] = __fmul_rn(y, y);
         }
         if (J.norm_next) {
           const float tot = warp_reduce<RB>(sq, lane);
@@ -1098,7 +1364,7 @@ struct Worker {
     if (wtid == 0) mbar_arrive(tc::smem_u32(&sh->acc_empty[buf]));
     ++n_acc;
     // cross-warp part of the per-row sums: add the four quarters in a fixed order
-    if (P.kind == G_O || (P.kind == G_DOWN && !J.dp && J.norm_next)) {
+    if (P.kind == G_O || (P.kind == G_DOWN && J.norm_next)) {
       // o product: MLP norm of this job; down product: the next job's first operand
       long long* ss = P.kind == G_O ? p.b.ss_m + (long long)jb * c.Rcap : p.b.ss_a + (long long)(jb + 1) * c.Rcap;
       for (int r = wtid; r < J.R; r += WORKERS)
@@ -1127,18 +1393,14 @@ struct Worker {
         *dst = make_float4(best, __int_as_float(bi), se, 0.f);
       }
     }
-    if (P.kind == G_HEAD || P.kind == G_O || (P.kind == G_DOWN && !J.dp)) worker_sync();  // tables reused by the next tile
+    if (P.kind == G_HEAD || P.kind == G_O || P.kind == G_DOWN) worker_sync();  // tables reused by the next tile
     return true;
   }
 
-  // skip candidate of state j (1-based) at row t: g[i-1][j-1]
-  // the same by row r = (j - 1) T + t of the step: state 1's candidates are the objective rows of the step
-  // before, the others row r - T ... of g, i.e. row r of the array that starts at g[i-1][0]
+  // skip candidate of state j (1-based) at row t, g[i-1][j-1], by row r = (j - 1) T + t of the step: state 1's candidates are the
+  // objective rows of the step before, the others row r - T ... of g, i.e. row r of the array that starts at g[i-1][0]
   __device__ __forceinline__ const float* skip_row(const Job& J, int r) const {
     return r < J.T ? J.x_im1 + r * J.x_im1_stride : J.g_prev + (long long)r * p.c.d;
-  }
-  __device__ __forceinline__ const float* skip_src(const Job& J, int j, int t) const {
-    return j == 1 ? J.x_im1 + t * J.x_im1_stride : J.g_prev + ((long long)(j - 1) * J.T + t) * p.c.d;
   }
 
   static constexpr double COS_FIX = 268435456.0;  // 2^28: sums up to 3e10 with 4e-9 resolution
@@ -1147,133 +1409,112 @@ struct Worker {
     asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(dst), "l"(q) : "memory");
   }
 
-  // This CTA's share of the three sums of Eq. 2 that do not involve a layer output, for the step of
-  // job `tgt` with `rows` candidate rows: x.s, s.s and x.x, where x = x_new[t] is that step's objective
-  // row and s the skip candidate of state j: x_old[t] for j = 1, else g[j - 1][t].  They are added
-  // to the job's accumulators as soon as the candidates exist, off the step's critical path.
-  __device__ void pre_sums(int tgt, int rows, int Tn, const float* x_new, const float* x_old, long long xs,
-                           long long xs_old, const float* g, bool fv, int f) {
+  // This CTA's share of the three sums of Eq. 2 that do not involve a layer output: x.s, s.s and x.x, where x is the step's
+  // objective row and s the skip candidate of the row's state.  They are added to the job's accumulators as soon as the
+  // candidates exist, off the step's critical path: a layer job does it while its o product is multiplied.  A deferred
+  // step's skip candidates also become the second row block of the next layer's operand (every CTA has finished this
+  // layer's q/k/v product, the last reader of that block, before its attention could start).
+  __device__ void pre_sums(const Job& J, int jb) {
     const Cfg& c = p.c;
-    RedTables* T = tables();
-    const int quarter = ww & 3, group = ww >> 2;
-    const int ncb = (rows + RB - 1) / RB;
-    const RowDiv rd(Tn);
-    for (int cb = group; cb < ncb; cb += 2) {
-      float pa[2 * RB], pb[RB];
-#pragma unroll
-      for (int k = 0; k < RB; ++k) {
-        const int r = cb * RB + k;
-        float xv = 0.f, sv = 0.f;
-        if (fv && r < rows) {
-          const int j = rd.div(r) + 1, t = rd.mod(r);
-          xv = __ldg(x_new + t * xs + f);
-          sv = __ldcg((j == 1 ? x_old + t * xs_old : g + ((long long)(j - 1) * Tn + t) * c.d) + f);
-        }
-        pa[k] = xv * sv;
-        pa[RB + k] = sv * sv;
-        pb[k] = xv * xv;
-      }
-      const float ta = warp_reduce<2 * RB>(pa, lane);
-      const float tb = warp_reduce<RB>(pb, lane);
-      const int r = cb * RB + (lane & (RB - 1));
-      if (lane < 2 * RB && r < rows) {
-        T->red[quarter][r][2 + lane / RB] = ta;
-        if (lane < RB) T->red[quarter][r][4] = tb;
-      }
-    }
-    worker_sync();
+    const int f_lo = __ldg(split_lo(S_D) + blockIdx.x);
+    const Slice sl(__ldg(split_lo(S_D) + blockIdx.x + 1) - f_lo, wtid);
+    const int f = f_lo + 4 * sl.q;
+    const int rows = (J.ell + (J.diag ? 1 : 0)) * J.T;
+    const RowDiv rd(J.T);
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 wq = zero;
+    if (sl.on && J.defer) wq = __ldg(reinterpret_cast<const float4*>(J.norm_next + f));
     unsigned long long* acc =
-        reinterpret_cast<unsigned long long*>(p.b.cosacc) + (long long)tgt * ((long long)(c.Rcap + MAX_ROWS) * 5);
-    for (int idx = wtid; idx < rows * 3; idx += WORKERS) {
-      const int r = idx / 3, k = 2 + idx % 3;
-      cos_add(acc + r * 5 + k, T->red[0][r][k] + T->red[1][r][k] + T->red[2][r][k] + T->red[3][r][k]);
+        reinterpret_cast<unsigned long long*>(p.b.cosacc) + (long long)jb * ((long long)(c.Rcap + MAX_ROWS) * 5);
+    const int passes = sl.passes(rows);
+#pragma unroll 1
+    for (int pass0 = 0; pass0 < passes; pass0 += PF) {
+      float4 x[PF], s[PF];
+#pragma unroll
+      for (int k = 0; k < PF; ++k) {
+        const int r = sl.r0 + (pass0 + k) * sl.step;
+        x[k] = zero;
+        s[k] = zero;
+        if (sl.on && r < rows) {
+          x[k] = __ldg(reinterpret_cast<const float4*>(J.x_i + rd.mod(r) * J.x_tok_stride + f));
+          s[k] = ld4(skip_row(J, r) + f);
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < PF; ++k) {
+        if (pass0 + k >= passes) break;
+        const int r = sl.r0 + (pass0 + k) * sl.step;
+        const bool ok = sl.on && r < rows;
+        if (ok && J.defer) st_bf16x4(p.b.xn_a + (long long)(c.BN + r) * c.d + f, s[k], wq);
+        float t[3] = {dot4(x[k], s[k]), dot4(s[k], s[k]), dot4(x[k], x[k])};
+        group_sum(t, sl.lq);
+        if (ok && sl.q == 0) {
+#pragma unroll
+          for (int e = 0; e < 3; ++e) cos_add(acc + r * 5 + 2 + e, t[e]);
+        }
+      }
     }
-    worker_sync();  // the tables are reused
   }
 
-  // ---- Eq. 2 step i over this CTA's slice of the d features (thread <-> feature as in the
-  // epilogue):
-  //   (1) this CTA's share of x.y and y.y goes to the job's fixed-point accumulators, publish;
-  //   (2) wait for every CTA, read the totals, decide (every CTA decides alike); the chosen row's
+  // ---- Eq. 2 step i over this CTA's slice of the d features (dealt by row as in epilogue_rows, which has added this CTA's
+  // share of x.y and y.y to the job's fixed-point accumulators and left the layer outputs in the staged rows):
+  //   (1) publish; (2) wait for every CTA, read the totals, decide (every CTA decides alike); the chosen row's
   //       sum of squares is also the next layer's norm factor;
-  //   (3) write this CTA's slice of the next layer's operand, publish;
+  //   (3) write this CTA's slice of the next layer's operand, publish (not when the step is deferred);
   //   (4) this CTA's slice of g[i][.].
   // The sums over the skip candidates (x.s, s.s, x.x) were added earlier: by a layer job while it waited
   // for its o product, by a select-only job at its start.
-  // from_epilogue: the down product's epilogue left the partials of this CTA in the tables and
-  // the thread's layer outputs / skip candidates of its first row block in keep_y / keep_s.
-  // Eq. 2 step, rows past the two worker groups' first blocks: they come from global memory, and their
-  // (row, feature) pairs are dealt to all worker threads -- with many rows (several objective rows per state) a
-  // thread per feature would walk its row blocks one dependent load after the other.  to_operand: the chosen
-  // rows, normed, as the next layer's operand; else as g[i][.] for the next step (row r of the step is
-  // g[i][j][t] with j T + t = r + T).  Only in the instantiation for long contexts and many rows.
-  __device__ __forceinline__ void spread_rows(const Job& J, int f_lo, int nf, int rows, bool to_operand) const {
-    const int d = p.c.d, r_rest = 2 * RB, n_rest = max(rows - r_rest, 0) * nf;
-    float* const g_out = J.g_next + (long long)J.T * d;
-    const int gf_lo = (J.M - 1) * J.T;                              // first row of state M, if the step has it
-    float* const gf_out = (J.g_final && rows > gf_lo) ? J.g_final : nullptr;
-#pragma unroll 4
-    for (int idx = wtid; idx < n_rest; idx += WORKERS) {
-      const int rq = idx / nf;
-      const int r = r_rest + rq, ff = f_lo + (idx - rq * nf);
-      const float y = sh->choice_row[r] ? __ldcg(p.b.Gbuf + (long long)r * d + ff) : __ldcg(skip_row(J, r) + ff);
-      if (to_operand) {
-        p.b.xn_a[(long long)r * d + ff] = __float2bfloat16_rn(y * __ldg(J.norm_next + ff));
-      } else {
-        __stcg(g_out + (long long)r * d + ff, y);
-        if (gf_out && r >= gf_lo) gf_out[(long long)(r - gf_lo) * d + ff] = y;
-      }
-    }
-  }
-
-  __device__ bool dp_step(const Job& J, int jb, bool from_epilogue, float (&keep_y)[RB], float (&keep_s)[RB]) {
+  // from_epilogue: keep_s holds the thread's skip candidate of the first pass.
+  __device__ bool dp_step(const Job& J, int jb, bool from_epilogue, float4& keep_s) {
     const Cfg& c = p.c;
-    RedTables* T = tables();
-    const int f_lo = __ldg(split_lo(S_D) + blockIdx.x), f_hi = __ldg(split_lo(S_D) + blockIdx.x + 1);
-    const int quarter = ww & 3, group = ww >> 2;
-    const int fl = feat_local(f_hi - f_lo, quarter, lane);   // a slice has at most 128 features (checked on the host)
-    const bool fv = fl >= 0;
-    const int f = f_lo + fl;
+    const int f_lo = __ldg(split_lo(S_D) + blockIdx.x);
+    const int n = __ldg(split_lo(S_D) + blockIdx.x + 1) - f_lo;   // at most 128 features (checked on the host)
+    const Slice sl(n, wtid);
+    const int f = f_lo + 4 * sl.q;
     const int n_states = J.ell + (J.diag ? 1 : 0);
     const int rows = n_states * J.T;
-    const int ncb = (rows + RB - 1) / RB;
-    unsigned long long* acc =
-        reinterpret_cast<unsigned long long*>(p.b.cosacc) + (long long)jb * ((long long)(c.Rcap + MAX_ROWS) * 5);
+    const int passes = sl.passes(rows);
     const RowDiv rd(J.T);
-    const float wn = (fv && J.norm_next) ? __ldg(J.norm_next + f) : 0.f;   // needed right after the decision
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    const unsigned long long* acc =
+        reinterpret_cast<const unsigned long long*>(p.b.cosacc) + (long long)jb * ((long long)(c.Rcap + MAX_ROWS) * 5);
+    float4 wn = zero;   // needed right after the decision
+    if (sl.on && J.norm_next && !J.defer) wn = __ldg(reinterpret_cast<const float4*>(J.norm_next + f));
     // (a layer job adds its sums over the skip candidates while it waits for its o product)
-    if (J.type == JOB_SELECT) pre_sums(jb, rows, J.T, J.x_i, J.x_im1, J.x_tok_stride, J.x_im1_stride, J.g_prev, fv, f);
-    if (!from_epilogue) {
-      // no layer ran for this CTA's features: only skip candidates exist
-#pragma unroll
-      for (int k = 0; k < RB; ++k) {
-        const int r = group * RB + k;
-        keep_y[k] = 0.f;
-        keep_s[k] = (fv && r < rows) ? __ldcg(skip_row(J, r) + f) : 0.f;
-      }
-    } else {
-      for (int idx = wtid; idx < J.R * 2; idx += WORKERS) {
-        const int r = idx >> 1, k = idx & 1;
-        cos_add(acc + r * 5 + k, T->red[0][r][k] + T->red[1][r][k] + T->red[2][r][k] + T->red[3][r][k]);
-      }
+    if (J.type == JOB_SELECT) pre_sums(J, jb);
+    if (!from_epilogue) {   // no layer ran for this CTA's features: only skip candidates exist
+      keep_s = zero;
+      if (sl.on && sl.r0 < rows) keep_s = ld4(skip_row(J, sl.r0) + f);
     }
     publish(F_DOWN, jb + 1);
     mark(T_DP_PUB);
-    // (2) once every CTA has added its share: read the totals, decide
+    // (2) once every CTA has added its share: a thread per row reads the totals
     if (!wait_all(F_DOWN, J.tgt[F_DOWN])) return false;
     mark(T_DP_ALL);
-    for (int idx = wtid; idx < rows * 5; idx += WORKERS)
-      T->cosv[idx / 5][idx % 5] = (double)(long long)__ldcg(acc + idx) * (1.0 / COS_FIX);
-    worker_sync();
-    if (wtid < n_states) {
-      const int j = wtid + 1;
+    float* tab = reinterpret_cast<float*>(scratch + c.stage_bytes);   // [2][MAX_ROWS]: the two cosines of each row
+    float app = 0.f, skp = 0.f, rs_app = 0.f, rs_skp = 0.f;
+    if (wtid < rows) {
+      float v[5];
+#pragma unroll
+      for (int e = 0; e < 5; ++e) v[e] = (float)((double)(long long)__ldcg(acc + wtid * 5 + e) * (1.0 / COS_FIX));
       // the sums are exact to the fixed-point step; the few operations on them run in float
-      float app = 0.f, skp = 0.f;
-      for (int t = 0; t < J.T; ++t) {
-        const double* v = T->cosv[(j - 1) * J.T + t];
-        const float nx = fmaxf(sqrtf((float)v[4]), 1e-12f);
-        app += (float)v[0] / (nx * fmaxf(sqrtf((float)v[1]), 1e-12f));
-        skp += (float)v[2] / (nx * fmaxf(sqrtf((float)v[3]), 1e-12f));
+      const float nx = fmaxf(sqrtf(v[4]), 1e-12f);
+      app = v[0] / (nx * fmaxf(sqrtf(v[1]), 1e-12f));
+      skp = v[2] / (nx * fmaxf(sqrtf(v[3]), 1e-12f));
+      rs_app = rsqrtf(v[1] / (float)c.d + c.eps);
+      rs_skp = rsqrtf(v[3] / (float)c.d + c.eps);
+      tab[wtid] = app;
+      tab[MAX_ROWS + wtid] = skp;
+    }
+    if (J.T > 1) worker_sync();
+    if (wtid < rows) {
+      const int j0 = rd.div(wtid), t0 = wtid - j0 * J.T, j = j0 + 1;
+      if (J.T > 1) {   // the state's mean over its rows (every row's thread sums it alike)
+        app = skp = 0.f;
+        for (int t = 0; t < J.T; ++t) {
+          app += tab[j0 * J.T + t];
+          skp += tab[MAX_ROWS + j0 * J.T + t];
+        }
       }
       const float s_app = app / (float)J.T, s_skip = skp / (float)J.T;
       int take = 0;
@@ -1281,13 +1522,9 @@ struct Worker {
         take = s_app > s_skip;
         if (J.forced && J.forced[j] != 255) take = (J.forced[j] == 0);
       }
-      sh->choice[j] = take;
-      for (int t = 0; t < J.T; ++t) sh->choice_row[(j - 1) * J.T + t] = take;
-      for (int t = 0; t < J.T; ++t) {
-        const double* v = T->cosv[(j - 1) * J.T + t];
-        sh->rs_next[(j - 1) * J.T + t] = rsqrtf((float)(take ? v[1] : v[3]) / (float)c.d + c.eps);
-      }
-      if (blockIdx.x == 0) {
+      sh->choice_row[wtid] = take;
+      sh->rs_next[wtid] = take ? rs_app : rs_skp;
+      if (blockIdx.x == 0 && t0 == 0) {
         J.D[j] = take ? s_app : s_skip;
         J.choice[j] = take ? 0 : 1;
         if (J.margin && j <= J.ell) J.margin[j] = s_app - s_skip;
@@ -1299,71 +1536,41 @@ struct Worker {
     }
     worker_sync();
     mark(T_DP_DECIDED);
-    // (3) the next layer's operand: the first block of rows comes from registers
-    float y16[RB];
+    // (3), (4): skip candidates past the first pass come from global memory, PF passes in flight; a step that hands the
+    // chosen rows on leaves them in the staged rows for (4)
+    float* const g_out = J.g_next + (long long)J.T * c.d + f;       // row r of the step is g[i][j][t] with j T + t = r + T
+    const int gf_lo = (J.M - 1) * J.T;                              // first row of state M, if the step has it
+    const bool to_operand = J.norm_next && !J.defer;
+    auto write_back = [&](bool operand, bool chosen) {
+#pragma unroll 1
+      for (int pass0 = 0; pass0 < passes; pass0 += PF) {
+        float4 s[PF];
 #pragma unroll
-    for (int k = 0; k < RB; ++k) {
-      const int r = group * RB + k;
-      y16[k] = 0.f;
-      if (fv && r < rows) y16[k] = sh->choice_row[r] ? keep_y[k] : keep_s[k];
-    }
-    if constexpr (TC) {
-      // (the instantiation for long contexts and many rows deals the rows past the first blocks to all threads)
-      if (J.norm_next && !J.defer) {
-        if (fv) {
-#pragma unroll
-          for (int k = 0; k < RB; ++k) {
-            const int r = group * RB + k;
-            if (r < rows) p.b.xn_a[(long long)r * c.d + f] = __float2bfloat16_rn(y16[k] * wn);
-          }
+        for (int k = 0; k < PF; ++k) {
+          const int r = sl.r0 + (pass0 + k) * sl.step;
+          s[k] = keep_s;
+          if (pass0 + k > 0 && sl.on && r < rows && !chosen && !sh->choice_row[r]) s[k] = ld4(skip_row(J, r) + f);
         }
-        spread_rows(J, f_lo, f_hi - f_lo, rows, true);
-      }
-    } else if (J.norm_next && fv && !J.defer) {
-      for (int cb = group; cb < ncb; cb += 2) {
 #pragma unroll
-        for (int k = 0; k < RB; ++k) {
-          const int r = cb * RB + k;
-          if (r < rows) {
-            const float y = cb == group ? y16[k]
-                                        : (sh->choice_row[r] ? __ldcg(p.b.Gbuf + (long long)r * c.d + f) : __ldcg(skip_row(J, r) + f));
-            p.b.xn_a[(long long)r * c.d + f] = __float2bfloat16_rn(y * wn);
+        for (int k = 0; k < PF; ++k) {
+          const int r = sl.r0 + (pass0 + k) * sl.step;
+          if (!sl.on || r >= rows) continue;
+          float4* at = reinterpret_cast<float4*>(stage() + r * n + 4 * sl.q);
+          const float4 y = chosen || sh->choice_row[r] ? *at : s[k];
+          if (operand) {
+            *at = y;
+            st_bf16x4(p.b.xn_a + (long long)r * c.d + f, y, wn);
+          } else {
+            __stcg(reinterpret_cast<float4*>(g_out + (long long)r * c.d), y);
+            if (J.g_final && r >= gf_lo) *reinterpret_cast<float4*>(J.g_final + (long long)(r - gf_lo) * c.d + f) = y;
           }
         }
       }
-    }
+    };
+    if (to_operand) write_back(true, false);
     if (!J.defer) publish(F_SELECT, jb + 1);   // (a deferred step's successor reads both candidates: nobody waits)
     mark(T_SEL_PUB);
-    // (4) g[i][.] for the next step (read back only by this thread: same feature in every step)
-    float* const g_out = J.g_next + (long long)J.T * c.d + f;
-    const int gf_lo = (J.M - 1) * J.T;                              // first row of state M, if the step has it
-    float* const gf_out = (J.g_final && rows > gf_lo) ? J.g_final + f : nullptr;
-    if constexpr (TC) {
-      if (fv) {
-#pragma unroll
-        for (int k = 0; k < RB; ++k) {
-          const int r = group * RB + k;
-          if (r < rows) {
-            __stcg(g_out + (long long)r * c.d, y16[k]);
-            if (gf_out && r >= gf_lo) gf_out[(long long)(r - gf_lo) * c.d] = y16[k];
-          }
-        }
-      }
-      spread_rows(J, f_lo, f_hi - f_lo, rows, false);
-    } else if (fv) {
-      for (int cb = group; cb < ncb; cb += 2) {
-#pragma unroll
-        for (int k = 0; k < RB; ++k) {
-          const int r = cb * RB + k;
-          if (r < rows) {   // row r of the step is g[i][j][t] with j T + t = r + T
-            const float y = cb == group ? y16[k]
-                                        : (sh->choice_row[r] ? __ldcg(p.b.Gbuf + (long long)r * c.d + f) : __ldcg(skip_row(J, r) + f));
-            __stcg(g_out + (long long)r * c.d, y);
-            if (gf_out && r >= gf_lo) gf_out[(long long)(r - gf_lo) * c.d] = y;
-          }
-        }
-      }
-    }
+    write_back(false, to_operand);
     return true;
   }
 
@@ -1386,10 +1593,290 @@ struct Worker {
     const int n_pbg = (Pn + 127) / 128;
     const int k_tot = J.uniform ? J.C + J.T : J.C;
     const int n_runs = (k_tot + c.run_len - 1) / c.run_len;
-    const int n_own = J.uniform ? 0 : (J.R + ATT_KEYS - 1) / ATT_KEYS;
-    const int n_chunks = n_runs + n_own;
-    const int n_ch = OWN_ONLY ? n_own : n_chunks;   // chunks this call deals out
-    const int n_items = c.nkv * n_ch * n_pbg;
+    const int n_own = J.uniform ? 0 : 1;
+    const int n_ch = OWN_ONLY ? n_own : n_runs + n_own;   // chunks per pair block this call deals out
+    const int n_items = c.nkv * n_pbg * n_ch;
+    // Items in the order (kv head, pair block, chunk): a CTA takes a contiguous range, so that it rotates a pair block's q
+    // once for all its chunks and fetches the next chunk's first tile under the tiles before it.
+    const int it0 = OWN_ONLY ? c.G - 1 - (int)blockIdx.x : n_items * (int)blockIdx.x / c.G;
+    const int it1 = OWN_ONLY ? n_items : n_items * ((int)blockIdx.x + 1) / c.G;
+    int pb = it0 / n_ch, ch = it0 - pb * n_ch;            // pair block (kv head x n_pbg + block), chunk
+    const int g8 = lane >> 2, c4 = lane & 3;
+    const long long kvld = c.kvd;
+    const int qkvd = c.qd + 2 * c.kvd;
+    const float qscale = rsqrtf((float)HD) * 1.4426950408889634f;
+    const RowDiv rdT(J.T);
+    const uint32_t tag = p.launch_tag | (uint32_t)(jb + 1);
+    // The cache does not depend on this layer's projections: the first K/V tile of this CTA's first
+    // item is on its way from HBM while the CTA waits for them.
+    constexpr int FILL = ATT_KEYS * (HD / 8) / WORKERS;   // 16-byte pieces of a tile per thread
+    static_assert(FILL * WORKERS == ATT_KEYS * (HD / 8), "tile pieces must divide among the workers");
+    uint4 pre_k[FILL], pre_v[FILL];
+    // pieces of the cache tile at k0 (keys of the run that ends at k_end) into the rolling registers, one tile ahead of their use
+    auto load_cache_tile = [&](int kvh, int k0, int k_end) {
+#pragma unroll
+      for (int e = 0; e < FILL; ++e) {
+        const int vv = wtid + e * WORKERS;
+        const int key = k0 + vv / (HD / 8), cv8 = vv % (HD / 8);
+        pre_k[e] = make_uint4(0, 0, 0, 0);
+        pre_v[e] = make_uint4(0, 0, 0, 0);
+        if (key < k_end && key < J.C) {   // positions this launch never writes
+          pre_k[e] = __ldcg(reinterpret_cast<const uint4*>(J.ck + (long long)key * kvld + kvh * HD + cv8 * 8));
+          pre_v[e] = __ldcg(reinterpret_cast<const uint4*>(J.cv + (long long)key * kvld + kvh * HD + cv8 * 8));
+        }
+      }
+    };
+    if (!OWN_ONLY && it0 < it1 && ch < n_runs) load_cache_tile(pb / n_pbg, ch * c.run_len, (ch + 1) * c.run_len);
+    // every row's q, k, v exist once all CTAs have published their slice of the projections
+    if (!OWN_ONLY) {
+      if (!wait_all(F_QKV, J.tgt[F_QKV])) return false;
+      mark(T_ATT_READY);
+    }
+    uint32_t qh[KS][4];
+    int p0 = 0, rr[2], hq[2], tq[2], sq[2];   // first pair of the warp; row, query head, position and state of the thread's rows
+    bool active = false, pv[2], new_q = true;
+    for (int it = it0; it < it1; it += OWN_ONLY ? c.G : 1) {
+      const int kvh = pb / n_pbg, pbg = pb - kvh * n_pbg;
+      const int chunk = OWN_ONLY ? n_runs : ch;
+      const bool own = chunk >= n_runs;
+      if (new_q) {
+        p0 = (pbg * 8 + ww) * 16;
+        active = p0 < Pn;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int pp = p0 + g8 + h * 8;
+          pv[h] = pp < Pn;
+          rr[h] = pv[h] ? pp / Gq : 0;
+          hq[h] = kvh * Gq + (pv[h] ? pp % Gq : 0);
+          sq[h] = rdT.div(rr[h]);
+          tq[h] = rr[h] - sq[h] * J.T;
+        }
+        // q fragments, rotated.  Element i of the first half pairs with element i + HD/2: one load
+        // of each gives the rotated values of both, i.e. the fragments of k-steps ks and ks + KS/2.
+        // all loads first (one trip to L2), then the rotation
+        float2 raw_lo[KS / 2][4], raw_hi[KS / 2][4];
+#pragma unroll
+        for (int ks = 0; ks < KS / 2; ++ks) {
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+#pragma unroll
+            for (int kh = 0; kh < 2; ++kh) {
+              raw_lo[ks][h + kh * 2] = make_float2(0.f, 0.f);
+              raw_hi[ks][h + kh * 2] = make_float2(0.f, 0.f);
+              if (active && pv[h]) {
+                const int i = ks * 16 + kh * 8 + c4 * 2;           // dims i, i + 1 of the first half
+                const float* qr = p.b.qkv + (long long)rr[h] * qkvd + hq[h] * HD;
+                raw_lo[ks][h + kh * 2] = __ldcg(reinterpret_cast<const float2*>(qr + i));
+                raw_hi[ks][h + kh * 2] = __ldcg(reinterpret_cast<const float2*>(qr + i + HALF));
+              }
+            }
+          }
+        }
+#pragma unroll
+        for (int ks = 0; ks < KS / 2; ++ks) {
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+#pragma unroll
+            for (int kh = 0; kh < 2; ++kh) {
+              const int i = ks * 16 + kh * 8 + c4 * 2;
+              const float2 lo2 = raw_lo[ks][h + kh * 2], hi2 = raw_hi[ks][h + kh * 2];
+              const float4 cs = *reinterpret_cast<const float4*>(p.b.rope + (long long)tq[h] * HALF + i);
+              const float2 v0 = make_float2((lo2.x * cs.x - hi2.x * cs.y) * qscale, (lo2.y * cs.z - hi2.y * cs.w) * qscale);
+              const float2 v1 = make_float2((hi2.x * cs.x + lo2.x * cs.y) * qscale, (hi2.y * cs.z + lo2.y * cs.w) * qscale);
+              qh[ks][h + kh * 2] = pack2(v0.x, v0.y);
+              qh[ks + KS / 2][h + kh * 2] = pack2(v1.x, v1.y);
+            }
+          }
+        }
+      }
+      mark(T_ATT_Q);
+      float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};
+      float o[NBLK][4];
+#pragma unroll
+      for (int nb = 0; nb < NBLK; ++nb) { o[nb][0] = o[nb][1] = o[nb][2] = o[nb][3] = 0.f; }
+
+      // own keys: from the first row of the state that the block's first row belongs to, up to the block's last row
+      int key_lo, key_hi;
+      if (!own) { key_lo = chunk * c.run_len; key_hi = min(k_tot, key_lo + c.run_len); }
+      else { key_lo = rdT.div(pbg * 128 / Gq) * J.T; key_hi = min(J.R, (pbg * 128 + 127) / Gq + 1); }
+      for (int key0 = key_lo; key0 < key_hi; key0 += ATT_KEYS) {
+        const int nkeys = min(ATT_KEYS, key_hi - key0);
+        worker_sync();  // previous tile consumed
+        // K/V tile: cache rows as they are; rows of this call rotated / rounded from the projections
+#pragma unroll
+        for (int e = 0; e < FILL; ++e) {
+          const int vv = wtid + e * WORKERS;
+          const int row = vv / (HD / 8), cv8 = vv % (HD / 8);
+          uint4 kk = make_uint4(0, 0, 0, 0), vq = make_uint4(0, 0, 0, 0);
+          if (row < nkeys) {
+            const int key = key0 + row;
+            const int new_row = own ? key : (J.uniform ? key - J.C : -1);
+            if (new_row < 0) {
+              kk = pre_k[e];
+              vq = pre_v[e];
+            } else {
+              const float* kr = p.b.qkv + (long long)new_row * qkvd + c.qd + kvh * HD;
+              const float* vr = kr + c.kvd;
+              const int d0 = cv8 * 8, i0 = d0 % HALF;
+              float ka[8], kb[8], vf[8];
+#pragma unroll
+              for (int e = 0; e < 8; e += 4) {
+                const float4 a4 = __ldcg(reinterpret_cast<const float4*>(kr + i0 + e));
+                const float4 b4 = __ldcg(reinterpret_cast<const float4*>(kr + i0 + HALF + e));
+                const float4 v4 = __ldcg(reinterpret_cast<const float4*>(vr + d0 + e));
+                ka[e] = a4.x; ka[e + 1] = a4.y; ka[e + 2] = a4.z; ka[e + 3] = a4.w;
+                kb[e] = b4.x; kb[e + 1] = b4.y; kb[e + 2] = b4.z; kb[e + 3] = b4.w;
+                vf[e] = v4.x; vf[e + 1] = v4.y; vf[e + 2] = v4.z; vf[e + 3] = v4.w;
+              }
+              float kro[8];
+#pragma unroll
+              for (int e = 0; e < 8; ++e) {
+                const float2 cs = p.b.rope[(long long)rdT.mod(new_row) * HALF + i0 + e];
+                kro[e] = d0 < HALF ? ka[e] * cs.x - kb[e] * cs.y : kb[e] * cs.x + ka[e] * cs.y;
+              }
+              const uint2 k01 = pack4(kro[0], kro[1], kro[2], kro[3]), k23 = pack4(kro[4], kro[5], kro[6], kro[7]);
+              const uint2 v01 = pack4(vf[0], vf[1], vf[2], vf[3]), v23 = pack4(vf[4], vf[5], vf[6], vf[7]);
+              kk = make_uint4(k01.x, k01.y, k23.x, k23.y);
+              vq = make_uint4(v01.x, v01.y, v23.x, v23.y);
+              if (J.uniform && pbg == 0) {  // this item owns the cache rows of its keys
+                *reinterpret_cast<uint4*>(J.ck + (long long)key * kvld + kvh * HD + cv8 * 8) = kk;
+                *reinterpret_cast<uint4*>(J.cv + (long long)key * kvld + kvh * HD + cv8 * 8) = vq;
+              }
+            }
+          }
+          *reinterpret_cast<uint4*>(k_s + row * LD + cv8 * 8) = kk;
+          *reinterpret_cast<uint4*>(v_s + row * LD + cv8 * 8) = vq;
+        }
+        if (!OWN_ONLY) {   // the next tile, of this chunk or the first of the next one, is in flight during this one's math
+          if (key0 + ATT_KEYS < key_hi) { if (!own) load_cache_tile(kvh, key0 + ATT_KEYS, key_hi); }
+          else if (it + 1 < it1 && ch + 1 < n_runs) load_cache_tile(kvh, (ch + 1) * c.run_len, (ch + 2) * c.run_len);
+          else if (it + 1 < it1 && ch + 1 >= n_ch) load_cache_tile((pb + 1) / n_pbg, 0, c.run_len);
+        }
+        worker_sync();
+        if (!active) continue;
+        // S = Q K^T.  The multiplies are issued in program order (volatile asm): the k-step is the outer loop,
+        // so that four independent accumulators alternate instead of eight dependent multiplies in a row.
+        float s[4][4];
+#pragma unroll
+        for (int nb = 0; nb < 4; ++nb) s[nb][0] = s[nb][1] = s[nb][2] = s[nb][3] = 0.f;
+#pragma unroll
+        for (int ks = 0; ks < KS; ++ks) {
+          uint32_t b0[4], b1[4];
+#pragma unroll
+          for (int nb = 0; nb < 4; ++nb) {
+            const bf16* kr = k_s + (nb * 8 + g8) * LD + c4 * 2 + ks * 16;
+            b0[nb] = *reinterpret_cast<const uint32_t*>(kr);
+            b1[nb] = *reinterpret_cast<const uint32_t*>(kr + 8);
+          }
+#pragma unroll
+          for (int nb = 0; nb < 4; ++nb) mma_16816(s[nb], qh[ks], b0[nb], b1[nb]);
+        }
+        float mx[2] = {-INFINITY, -INFINITY};
+#pragma unroll
+        for (int nb = 0; nb < 4; ++nb) {
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const int h = e >> 1;
+            const int key = key0 + nb * 8 + c4 * 2 + (e & 1);
+            bool vis = pv[h] && key < key_hi;
+            if (own) vis = vis && (rdT.div(key) == sq[h]) && key <= rr[h];
+            else if (J.uniform) vis = vis && key <= J.C + rr[h];
+            if (!vis) s[nb][e] = -INFINITY;
+            mx[h] = fmaxf(mx[h], s[nb][e]);
+          }
+        }
+        float corr[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 1));
+          mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 2));
+          const float m_new = fmaxf(m[h], mx[h]);
+          corr[h] = (m_new == -INFINITY) ? 1.f : exp2f(m[h] - m_new);
+          m[h] = m_new;
+        }
+        float rsum[2] = {0.f, 0.f};
+#pragma unroll
+        for (int nb = 0; nb < 4; ++nb) {
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const int h = e >> 1;
+            const float pe = (s[nb][e] == -INFINITY) ? 0.f : exp2f(s[nb][e] - m[h]);
+            s[nb][e] = pe;
+            rsum[h] += pe;
+          }
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          rsum[h] += __shfl_xor_sync(0xffffffffu, rsum[h], 1);
+          rsum[h] += __shfl_xor_sync(0xffffffffu, rsum[h], 2);
+          l[h] = l[h] * corr[h] + rsum[h];
+        }
+#pragma unroll
+        for (int nb = 0; nb < NBLK; ++nb) {
+          o[nb][0] *= corr[0]; o[nb][1] *= corr[0];
+          o[nb][2] *= corr[1]; o[nb][3] *= corr[1];
+        }
+#pragma unroll
+        for (int k2 = 0; k2 < 2; ++k2) {
+          uint32_t ph[4];
+          ph[0] = pack2(s[2 * k2][0], s[2 * k2][1]);
+          ph[1] = pack2(s[2 * k2][2], s[2 * k2][3]);
+          ph[2] = pack2(s[2 * k2 + 1][0], s[2 * k2 + 1][1]);
+          ph[3] = pack2(s[2 * k2 + 1][2], s[2 * k2 + 1][3]);
+          const int mrow = k2 * 16 + (lane & 7) + ((lane >> 3) & 1) * 8;
+          const int mcol = (lane >> 4) * 8;
+#pragma unroll
+          for (int nb = 0; nb < NBLK; nb += 8) {   // four fragment loads in flight, then their eight multiplies
+            uint32_t vb[4][4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+              ldmatrix_x4_trans(tc::smem_u32(v_s + mrow * LD + (nb + 2 * q) * 8 + mcol), vb[q][0], vb[q][1], vb[q][2], vb[q][3]);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              mma_16816(o[nb + 2 * q], ph, vb[q][0], vb[q][1]);
+              mma_16816(o[nb + 2 * q + 1], ph, vb[q][2], vb[q][3]);
+            }
+          }
+        }
+      }
+      mark(T_ATT_TILES);
+      if (active) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          if (!pv[h]) continue;
+          // Every 8-byte store carries its own tag, so the merge needs no flag and no fence: it reads the
+          // partial results themselves until every piece shows this job's tag (8-byte accesses are single
+          // copies).  Values as bf16: the merged row is rounded to bf16 for the o product anyway.
+          const long long idx = ((long long)rr[h] * c.nq + hq[h]) * c.chunk_cap + chunk;
+          uint2* pa = p.b.att_acc + idx * (HD / 2) + c4;
+#pragma unroll
+          for (int nb = 0; nb < NBLK; ++nb) __stcg(pa + nb * 4, make_uint2(pack2(o[nb][2 * h], o[nb][2 * h + 1]), tag));
+          if (c4 == 0) __stcg(p.b.att_ml + idx, make_uint4(__float_as_uint(m[h]), tag, __float_as_uint(l[h]), tag));
+        }
+      }
+      if (OWN_ONLY) pb += c.G;
+      else if (++ch == n_ch) { ch = 0; ++pb; }
+      new_q = OWN_ONLY || ch == 0;
+    }
+    return true;
+  }
+
+  // The form for launches whose pairs fit one block (the instantiation without MR): an item is a chunk.  With the loop of the
+  // other form, which carries q and the next chunk's tile from item to item, a layer of one to twelve rows takes 1 us longer.
+  __device__ bool attention_one(const Job& J, int jb) {
+    const Cfg& c = p.c;
+    constexpr int KS = HD / 16;
+    constexpr int NBLK = HD / 8;
+    constexpr int LD = HD + 8;
+    constexpr int HALF = HD / 2;
+    bf16* k_s = reinterpret_cast<bf16*>(scratch);
+    bf16* v_s = k_s + ATT_KEYS * LD;
+    const int Gq = c.nq / c.nkv;
+    const int Pn = J.R * Gq;
+    const int k_tot = J.uniform ? J.C + J.T : J.C;
+    const int n_runs = (k_tot + c.run_len - 1) / c.run_len;
+    const int n_chunks = n_runs + (J.uniform ? 0 : 1);
+    const int n_items = c.nkv * n_chunks;
     const int g8 = lane >> 2, c4 = lane & 3;
     const long long kvld = c.kvd;
     const int qkvd = c.qd + 2 * c.kvd;
@@ -1402,9 +1889,9 @@ struct Worker {
     static_assert(FILL * WORKERS == ATT_KEYS * (HD / 8), "tile pieces must divide among the workers");
     uint4 pre_k[FILL], pre_v[FILL];
     bool pre_ok = false;
-    if (!OWN_ONLY && (int)blockIdx.x < n_items) {
-      const int chunk = ((int)blockIdx.x / n_pbg) % n_chunks;
-      const int kvh = (int)blockIdx.x / (n_pbg * n_chunks);
+    if ((int)blockIdx.x < n_items) {
+      const int chunk = (int)blockIdx.x % n_chunks;
+      const int kvh = (int)blockIdx.x / n_chunks;
       if (chunk < n_runs) {
         const int key_lo = chunk * c.run_len;
         pre_ok = true;
@@ -1422,16 +1909,13 @@ struct Worker {
       }
     }
     // every row's q, k, v exist once all CTAs have published their slice of the projections
-    if (!OWN_ONLY) {
-      if (!wait_all(F_QKV, J.tgt[F_QKV])) return false;
-      mark(T_ATT_READY);
-    }
-    for (int it = OWN_ONLY ? c.G - 1 - (int)blockIdx.x : (int)blockIdx.x; it < n_items; it += c.G) {
-      const int pbg = it % n_pbg;
-      const int chunk = (OWN_ONLY ? n_runs : 0) + (it / n_pbg) % n_ch;
-      const int kvh = it / (n_pbg * n_ch);
+    if (!wait_all(F_QKV, J.tgt[F_QKV])) return false;
+    mark(T_ATT_READY);
+    for (int it = (int)blockIdx.x; it < n_items; it += c.G) {
+      const int chunk = it % n_chunks;
+      const int kvh = it / n_chunks;
       const bool own = chunk >= n_runs;
-      const int p0 = (pbg * 8 + ww) * 16;
+      const int p0 = ww * 16;
       const bool active = p0 < Pn;
       int rr[2], hq[2], tq[2], sq[2];   // row, query head, position and state of the row
       bool pv[2];
@@ -1492,7 +1976,7 @@ struct Worker {
 
       int key_lo, key_hi;
       if (!own) { key_lo = chunk * c.run_len; key_hi = min(k_tot, key_lo + c.run_len); }
-      else { key_lo = (chunk - n_runs) * ATT_KEYS; key_hi = min(J.R, key_lo + ATT_KEYS); }
+      else { key_lo = 0; key_hi = J.R; }
       // cache pieces of the tile at k0 into the rolling registers (issued one tile ahead of their use)
       auto load_cache_tile = [&](int k0) {
 #pragma unroll
@@ -1547,7 +2031,7 @@ struct Worker {
               const uint2 v01 = pack4(vf[0], vf[1], vf[2], vf[3]), v23 = pack4(vf[4], vf[5], vf[6], vf[7]);
               kk = make_uint4(k01.x, k01.y, k23.x, k23.y);
               vq = make_uint4(v01.x, v01.y, v23.x, v23.y);
-              if (J.uniform && pbg == 0) {  // this item owns the cache rows of its keys
+              if (J.uniform) {  // this item owns the cache rows of its keys
                 *reinterpret_cast<uint4*>(J.ck + (long long)key * kvld + kvh * HD + cv8 * 8) = kk;
                 *reinterpret_cast<uint4*>(J.cv + (long long)key * kvld + kvh * HD + cv8 * 8) = vq;
               }
@@ -2000,7 +2484,7 @@ struct Worker {
     const Cfg& c = p.c;
     const int k_tot = J.uniform ? J.C + J.T : J.C;
     const int n_runs = (k_tot + c.run_len - 1) / c.run_len;
-    const int n_chunks = n_runs + (J.uniform ? 0 : (J.R + ATT_KEYS - 1) / ATT_KEYS);
+    const int n_chunks = n_runs + (J.uniform ? 0 : 1);
     const uint32_t tag = p.launch_tag | (uint32_t)(jb + 1);
     const uint32_t n_poll = 2u * sh->wait_slow;
     bool all_ok = true;
@@ -2028,6 +2512,7 @@ struct Worker {
         return __all_sync(0xffffffffu, ok);
       };
       auto poll_trip = [&](int ch0, bool with_ml) -> bool {
+#pragma unroll 1
         for (uint32_t it = 0; it < n_poll; ++it) {
           if (load_trip(ch0, with_ml)) return true;
           if ((it & 15u) == 15u && aborted(p.ctl, sh)) return false;
@@ -2036,16 +2521,19 @@ struct Worker {
         raise_abort(p.ctl, sh, true);
         return false;
       };
-      if (!poll_trip(0, true)) { all_ok = false; break; }
-      const float m0 = __uint_as_float(v0.x), m1 = __uint_as_float(v1.x);
-      const float mx = warp_max(fmaxf(m0, m1));
-      const float w0 = m0 == -INFINITY ? 0.f : exp2f(m0 - mx);
-      const float w1 = m1 == -INFINITY ? 0.f : exp2f(m1 - mx);
-      const float den = warp_sum(w0 * __uint_as_float(v0.z) + w1 * __uint_as_float(v1.z));
+      float w0 = 0.f, w1 = 0.f, den = 1.f;
       float num[4] = {0.f, 0.f, 0.f, 0.f};
       bool ok = true;
+#pragma unroll 1
       for (int ch0 = 0; ch0 < n_chunks; ch0 += MB) {
-        if (ch0 > 0 && !poll_trip(ch0, false)) { ok = false; break; }
+        if (!poll_trip(ch0, ch0 == 0)) { ok = false; break; }
+        if (ch0 == 0) {
+          const float m0 = __uint_as_float(v0.x), m1 = __uint_as_float(v1.x);
+          const float mx = warp_max(fmaxf(m0, m1));
+          w0 = m0 == -INFINITY ? 0.f : exp2f(m0 - mx);
+          w1 = m1 == -INFINITY ? 0.f : exp2f(m1 - mx);
+          den = warp_sum(w0 * __uint_as_float(v0.z) + w1 * __uint_as_float(v1.z));
+        }
 #pragma unroll
         for (int e = 0; e < MB; ++e) {
           const int ch = ch0 + e;
@@ -2108,9 +2596,7 @@ struct Worker {
   __device__ bool run() {
     const Cfg& c = p.c;
     const TileDesc* tiles = reinterpret_cast<const TileDesc*>(p.tabs + c.tiles_off);
-    float keep_y[RB], keep_s[RB];
-#pragma unroll
-    for (int k = 0; k < RB; ++k) { keep_y[k] = 0.f; keep_s[k] = 0.f; }
+    float4 keep_s = make_float4(0.f, 0.f, 0.f, 0.f);   // the thread's skip candidate of the first pass over an Eq. 2 step's rows
     for (int jb = 0; jb < p.n_jobs; ++jb) {
       // the job descriptor goes to shared memory and from there into a local copy: its fields
       // must not look as if a store to global memory could change them
@@ -2123,41 +2609,56 @@ struct Worker {
       const Job J = *reinterpret_cast<const Job*>(sh->job_words);
       n_mark = jb;
       mark(T_START);
-      if (J.type == JOB_SELECT) {
-        if (!dp_step(J, jb, false, keep_y, keep_s)) return false;
-        continue;
-      }
       if (J.type == JOB_HEAD) {
         Phase P;
         P.init(p, J, 0);
-        for (int t = 0; t < P.n_tiles; ++t)
-          if (!epilogue(J, jb, P, tiles[P.tile0 + t], t, keep_y, keep_s)) return false;
+        for (int t = 0; t < P.n_tiles; ++t) {
+          if constexpr (FW) {
+            if (!epilogue_fwd(J, jb, P, tiles[P.tile0 + t], t)) return false;
+          } else if constexpr (MR) {
+            if (!epilogue_head(J, jb, tiles[P.tile0 + t], t)) return false;
+          }
+        }
+        if (P.n_tiles > 0) ++n_prod;
         if (!head_merge(J, jb)) return false;
         mark(T_HEAD);
         continue;
       }
       if (J.prep) prep(J, jb + 1);
-      for (int ph = 0; ph < 4; ++ph) {
+      bool from_epilogue = false;
+#pragma unroll 1
+      for (int ph = 0; ph < (J.type == JOB_LAYER ? 4 : 0); ++ph) {
         Phase P;
         P.init(p, J, ph);
-        if (ph == G_O && J.dp) {
+        if (!FW && ph == G_O && J.dp) {
           // idle time (the o product is being multiplied): this CTA's share of the sums of this job's
           // Eq. 2 step over the skip candidates, which the previous step left in g
-          const int f_lo = __ldg(split_lo(S_D) + blockIdx.x), f_hi = __ldg(split_lo(S_D) + blockIdx.x + 1);
-          const int fl = feat_local(f_hi - f_lo, ww & 3, lane);
-          pre_sums(jb, (J.ell + (J.diag ? 1 : 0)) * J.T, J.T, J.x_i, J.x_im1, J.x_tok_stride, J.x_im1_stride, J.g_prev, fl >= 0,
-                   f_lo + fl);
+          pre_sums(J, jb);
         }
-        for (int t = 0; t < P.n_tiles; ++t)
-          if (!epilogue(J, jb, P, tiles[P.tile0 + t], t, keep_y, keep_s)) return false;
+        if constexpr (FW) {
+          for (int t = 0; t < P.n_tiles; ++t)
+            if (!epilogue_fwd(J, jb, P, tiles[P.tile0 + t], t)) return false;
+        } else if (ph == G_O || ph == G_DOWN) {
+          if (P.n_tiles > 0 && !epilogue_rows(J, jb, ph, tiles[P.tile0], keep_s)) return false;   // (a slice is one tile)
+        } else {
+          for (int t = 0; t < P.n_tiles; ++t)
+            if (!epilogue_features(J, jb, P, tiles[P.tile0 + t], t)) return false;
+        }
+        if (P.n_tiles > 0) ++n_prod;
         mark(ph == G_QKV ? T_QKV : (ph == G_O ? T_O : (ph == G_GU ? T_GU : T_DOWN)));
         if (ph == G_QKV) {
+          // (the tiles that TMA brings next lie where epilogues and the Eq. 2 step have read and written)
+          if constexpr (TC) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
           publish(F_QKV, jb + 1);
           if constexpr (TC) {   // (only launched for searches over long contexts: no forward-pass jobs)
             if (!attention_tc(J, jb)) return false;
             if (!attention_partials<true>(J, jb)) return false;
           } else {
-            if (!attention_partials(J, jb)) return false;
+            if constexpr (MR) {
+              if (!attention_partials(J, jb)) return false;
+            } else {
+              if (!attention_one(J, jb)) return false;
+            }
           }
           mark(T_ATT_PUB);
           if (!attention_merge(J, jb)) return false;
@@ -2167,14 +2668,14 @@ struct Worker {
         } else if (ph == G_GU) {
           publish(F_GU, jb + 1);
         } else {
-          if (J.dp) {
-            if (!dp_step(J, jb, P.n_tiles > 0, keep_y, keep_s)) return false;
-          } else {
-            publish(F_DOWN, jb + 1);
-          }
-          mark(T_DP_DONE);
+          from_epilogue = P.n_tiles > 0;
+          if (!J.dp) publish(F_DOWN, jb + 1);
         }
       }
+      if constexpr (!FW) {
+        if ((J.dp || J.type == JOB_SELECT) && !dp_step(J, jb, from_epilogue, keep_s)) return false;
+      }
+      mark(T_DP_DONE);
     }
     return true;
   }
@@ -2186,7 +2687,7 @@ constexpr int REGS_WORKER = (THREADS * 168 - 128 * REGS_SPECIAL) / 256 / 8 * 8;
 static_assert(THREADS == 384 && WORKER_T0 == 128, "register split assumes one special and two worker warp groups");
 static_assert(128 * REGS_SPECIAL + 256 * REGS_WORKER <= THREADS * 168, "register pool of the CTA");
 
-template <bool TR, int HD, bool TC>
+template <bool TR, int HD, int KIND>
 __global__ void __launch_bounds__(THREADS, 1)
 engine_kernel(const __grid_constant__ CUtensorMap map_xn_a, const __grid_constant__ CUtensorMap map_attn,
               const __grid_constant__ CUtensorMap map_xn_m, const __grid_constant__ CUtensorMap map_act,
@@ -2218,6 +2719,7 @@ engine_kernel(const __grid_constant__ CUtensorMap map_xn_a, const __grid_constan
     sh.wait_fast = p.wait_fast;
     sh.wait_slow = p.wait_slow;
     sh.a_issued = 0;
+    sh.b_seen = 0;
     sh.flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -2249,7 +2751,7 @@ engine_kernel(const __grid_constant__ CUtensorMap map_xn_a, const __grid_constan
     }
   } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS_WORKER));
-    Worker<TR, HD, TC> w{p, &sh, scratch, tmem_base, (int)threadIdx.x - WORKER_T0, warp - 4, lane, 0u, 0};
+    Worker<TR, HD, KIND> w{p, &sh, scratch, tmem_base, (int)threadIdx.x - WORKER_T0, warp - 4, lane, 0u, 0, 0};
     w.run();
   }
 
