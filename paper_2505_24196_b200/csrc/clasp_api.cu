@@ -1145,7 +1145,7 @@ int engine_launch(clasp_ctx* ctx, int Rmax, int head_off, clasp::SetupArgs setup
   void* args[] = {(void*)&bm->second[0], (void*)&bm->second[1], (void*)&bm->second[2], (void*)&bm->second[3],
                   (void*)&hm->second[0], (void*)&bm->second[4], (void*)&bm->second[5], (void*)&bm->second[6],
                   (void*)&bm->second[7], (void*)&hm->second[1], (void*)&bm->second[8], (void*)&bm->second[9], (void*)&P};
-  // (pairs of more than one block: their attention carries q from chunk to chunk, 20 us of a 150 us layer at 192 pairs over 2048
+  // (pairs of more than one block: their attention carries q from chunk to chunk, 9 us of a 157 us layer at 192 pairs over 2048
   // positions; of one block, and the epilogues of a forward's few rows: figures at attention_one and epilogue_fwd)
   const int kind = att_tc ? pk::K_TC : (att_pairs > 128 ? pk::K_MANY : (search_ctx >= 0 ? pk::K_SEARCH : pk::K_FORWARD));
   const void* kern = ctx->e_kernel[2 * kind + (ctx->e_trace ? 1 : 0)];
