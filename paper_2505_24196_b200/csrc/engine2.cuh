@@ -1230,8 +1230,9 @@ struct Worker {
 
   // ---- epilogue of one accumulator in the instantiation for forward passes of few rows: tile td of product P.kind.
   // Thread (quarter q, lane) owns feature td.f0 + 32 q + lane; the two warps of a quarter take alternating blocks of RB rows
-  // (accumulator columns).  Per-row sums over the CTA's features go through RowTables: one entry per (quarter, row).  Of one
-  // to sixteen rows a layer takes 1.4 us less this way than through epilogue_rows; the sums are the same bits.
+  // (accumulator columns).  Per-row sums over the CTA's features go through RowTables: one entry per (quarter, row).  A layer
+  // of one to five rows takes 0.8 us less this way than through epilogue_rows (verification of five rows, 8B: 3247 -> 3221 us);
+  // the sums are the same bits.
   __device__ bool epilogue_fwd(const Job& J, int jb, const Phase& P, const TileDesc& td, int tile_no) {
     const Cfg& c = p.c;
     RowTables* T = reinterpret_cast<RowTables*>(scratch);
@@ -1862,7 +1863,8 @@ struct Worker {
   }
 
   // The form for launches whose pairs fit one block (the instantiation without MR): an item is a chunk.  With the loop of the
-  // other form, which carries q and the next chunk's tile from item to item, a layer of one to twelve rows takes 1 us longer.
+  // other form, which carries q and the next chunk's tile from item to item, a layer of twelve rows takes 0.6 us longer (8B
+  // search at 512 positions 3073 -> 3100 us).
   __device__ bool attention_one(const Job& J, int jb) {
     const Cfg& c = p.c;
     constexpr int KS = HD / 16;
@@ -2522,17 +2524,28 @@ struct Worker {
         return false;
       };
       float w0 = 0.f, w1 = 0.f, den = 1.f;
+      auto weights = [&]() {
+        const float m0 = __uint_as_float(v0.x), m1 = __uint_as_float(v1.x);
+        const float mx = warp_max(fmaxf(m0, m1));
+        w0 = m0 == -INFINITY ? 0.f : exp2f(m0 - mx);
+        w1 = m1 == -INFINITY ? 0.f : exp2f(m1 - mx);
+        den = warp_sum(w0 * __uint_as_float(v0.z) + w1 * __uint_as_float(v1.z));
+      };
       float num[4] = {0.f, 0.f, 0.f, 0.f};
       bool ok = true;
+      // (the first trip outside the loop is the faster form where it is the only one: 8B search at 512 positions 3077 -> 3067 us;
+      // with many rows the smaller code is: 2048 positions, T = 4 4440 -> 4298)
+      if constexpr (!MR && !TC) {
+        if (!poll_trip(0, true)) { all_ok = false; break; }
+        weights();
+      }
 #pragma unroll 1
       for (int ch0 = 0; ch0 < n_chunks; ch0 += MB) {
-        if (!poll_trip(ch0, ch0 == 0)) { ok = false; break; }
-        if (ch0 == 0) {
-          const float m0 = __uint_as_float(v0.x), m1 = __uint_as_float(v1.x);
-          const float mx = warp_max(fmaxf(m0, m1));
-          w0 = m0 == -INFINITY ? 0.f : exp2f(m0 - mx);
-          w1 = m1 == -INFINITY ? 0.f : exp2f(m1 - mx);
-          den = warp_sum(w0 * __uint_as_float(v0.z) + w1 * __uint_as_float(v1.z));
+        if constexpr (!MR && !TC) {
+          if (ch0 > 0 && !poll_trip(ch0, false)) { ok = false; break; }
+        } else {
+          if (!poll_trip(ch0, ch0 == 0)) { ok = false; break; }
+          if (ch0 == 0) weights();
         }
 #pragma unroll
         for (int e = 0; e < MB; ++e) {
