@@ -434,23 +434,27 @@ int gemm_wide(clasp_ctx* ctx, const GemmCall& g) {
     f_tiles += p.f_tiles[m];
   }
   p.tiles = f_tiles * p.row_tiles;
-  // Pairs at work: one per two SMs, each with at least eight chunks.  Four chunks make the small products slower (down
-  // product of d_ffn 3584, 129 - 500 rows: 50 us against 39), sixteen faster (34 - 37; o product of the 8B shape, 129 rows,
-  // 35 against 43, the other 8B products the same).
-  int W = ctx->num_sms / 2;
-  const long long units = (long long)p.tiles * p.kc;
-  if (units / 8 < W) W = units / 8 < 1 ? 1 : (int)(units / 8);
-  // What whole waves of tiles leave over is split over K where that saves a pair at least SPLIT_MIN_SAVED chunks: a chunk
-  // takes 0.27 - 0.31 us, the partial sums of a split tile (131 KB per part and CTA, written, counted and read back) 16 us
-  // and 0.1 us per chunk.  Single launches on the 8B shape, us, left-over tiles split / together with one whole wave / nothing:
-  //    257 rows   q/k/v  44 /  45 /  33   o  43 /  43 /  35   gate/up 215 / 109 / 105   down  72 /  71 /  84
-  //   1300 rows          60 /  60 /  60      66 /  71 /  60           271 / 232 / 236        136 / 174 / 173
-  //   1999 rows          90 /  91 /  89      74 /  86 /  68           333 / 307 / 314        183 / 247 / 193
-  // and 1999 rows in a loop under the power cap 99 / 102 / 95, 81 / 86 / 71, 409 / 388 / 386, 219 / 299 / 213.  So it pays
-  // for down products whose last wave is up to half full (257 rows save 127 chunks, 1300 rows 157; 1999 rows would save 60).
-  constexpr int SPLIT_MIN_SAVED = 100;
+  const int W = ctx->num_sms / 2;   // pairs of CTAs, one per two SMs
+  // What whole waves of tiles leave over goes to one pair each, or is split over K: `parts` pairs per tile, at most MAX_PARTS,
+  // so that a part never crosses a tile; of more than half a wave, all pairs share the row of (tile, chunk) units.  A chunk
+  // takes 0.27 - 0.31 us; a part costs its 131 KB per CTA, written, and read by the pair that finishes the tile, one part after
+  // the other (about 3 us each, hidden as far as the multiplies of that pair's next whole tile reach).  So the parts are few,
+  // and the split has to save a pair enough chunks: 60 with a whole tile behind it, 100 alone (K of 4096, at most 48, never
+  // does: 3 - 5 % from 769 rows on, but 116 -> 123 us for gate/up at 257).  Single launches, us, nothing split / the left-over
+  // tiles over all 74 pairs / together with one whole wave / as decided here, in turn on one box:
+  //   8192 wide, 28672 of FFN (K 8192, 8192, 8192, 28672)         4096 wide, 14336 of FFN: down (the others stay whole)
+  //    200 rows  gate/up  217 / 295 / 197 / 192   down 148 / 115 / 119 / 109      129 rows  114 /  77 /  77 /  69
+  //    400 rows  q/k/v     98 /  89 /  82 /  74   gate/up 340 / 375 / 316 / 312   257 rows   86 /  76 /  74 /  70
+  //   1000 rows  q/k/v    175 / 146 / 149 / 142   down 374 / 382 / 519 / 374     1300 rows  166 / 129 / 172 / 131
+  //   1700 rows  o        232 / 331 / 202 / 198   down 729 / 608 / 637 / 604     1700 rows  172 / 150 / 180 / 150
+  //   2000 rows  q/k/v    306 / 304 / 275 / 271   o    257 / 255 / 241 / 233     3400 rows  357 / 396 / 304 / 304
+  constexpr int MAX_PARTS = 4;
   const int full = p.tiles / W, left = p.tiles - full * W;
-  p.sk_tiles = left > 0 && p.kc - (int)((long long)left * p.kc / W) >= SPLIT_MIN_SAVED ? left : 0;
+  const int parts = left > 0 ? std::min(W / left, MAX_PARTS) : 0;
+  p.sk_pairs = parts >= 2 ? left * parts : W;
+  const int saved = p.kc - (int)((long long)left * p.kc / p.sk_pairs);
+  const int worth = parts < 2 ? std::max(100, p.kc * 2 / 5) : (full > 0 ? 60 : 100);
+  p.sk_tiles = left > 0 && saved >= worth ? left : 0;
   if (p.sk_tiles * 2 > MAX_COUNTERS || (size_t)W * 4 * wd::SLOT_FLOATS > PARTIAL_FLOATS) p.sk_tiles = 0;
   p.epi = g.epi;
   p.yf = g.yf; p.ldy = g.ldy; p.resid = g.resid; p.ldr = g.ldr; p.yo = (bf16*)g.yo; p.ldo = g.ldo;

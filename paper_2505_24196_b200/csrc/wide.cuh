@@ -32,7 +32,7 @@ struct GemmParams {
   int n_mats;              // 1..3 matrices stacked along the features
   int N[3], f_tiles[3], col_off[3];
   int row_tiles, tiles;    // 256-row tiles; all tiles
-  int sk_tiles;            // tiles [0, sk_tiles) are split over K among all pairs, the others go to one pair each
+  int sk_tiles, sk_pairs;  // tiles [0, sk_tiles) are split over K among the first sk_pairs pairs, the others go to one pair each
   int dual, epi;
   float* yf;
   long long ldy;
@@ -164,16 +164,17 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32
 
 // ------------------------------------------------------------------ the products
 // Work list of a pair w of W: first its share of the tiles that are split over K -- all their (tile, chunk) units in one
-// row, cut into W equal ranges --, then whole tiles w, w + W, ...  The split part, if any, is what whole waves of tiles leave over.
+// row, cut into sk_pairs equal ranges --, then whole tiles w, w + W, ...  The split part, if any, is what whole waves of tiles
+// leave over.
 struct Items {
   long long u, u1;
   int dp, W;
-  __device__ __forceinline__ static long long start(const GemmParams& p, int w, int W) {
-    return (long long)p.sk_tiles * p.kc * w / W;
+  __device__ __forceinline__ static long long start(const GemmParams& p, int w) {
+    return (long long)p.sk_tiles * p.kc * min(w, p.sk_pairs) / p.sk_pairs;
   }
   __device__ __forceinline__ Items(const GemmParams& p, int w, int W_) : W(W_) {
-    u = start(p, w, W_);
-    u1 = start(p, w + 1, W_);
+    u = start(p, w);
+    u1 = start(p, w + 1);
     dp = p.sk_tiles + w;
   }
   __device__ __forceinline__ bool next(const GemmParams& p, int& tile, int& kb, int& ke) {
@@ -349,12 +350,12 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ C
         // a part of the tile: partial sums to the workspace; the pair that comes last adds all parts in pair order
         const long long t0 = (long long)tile * p.kc, t1 = t0 + p.kc;
         const long long U = (long long)p.sk_tiles * p.kc;
-        first = (int)(t0 * W / U);
-        while (Items::start(p, first + 1, W) <= t0) ++first;
-        while (Items::start(p, first, W) > t0) --first;
+        first = (int)(t0 * p.sk_pairs / U);
+        while (Items::start(p, first + 1) <= t0) ++first;
+        while (Items::start(p, first) > t0) --first;
         last = first;
-        while (Items::start(p, last + 1, W) < t1) ++last;
-        float* slot = p.partial + ((long long)blockIdx.x * 2 + (Items::start(p, w, W) >= t0 ? 0 : 1)) * SLOT_FLOATS;
+        while (Items::start(p, last + 1) < t1) ++last;
+        float* slot = p.partial + ((long long)blockIdx.x * 2 + (Items::start(p, w) >= t0 ? 0 : 1)) * SLOT_FLOATS;
 #pragma unroll 1
         for (int c = half * (TN / 2); c < (half + 1) * (TN / 2); c += 32) {
           float v[32];
@@ -385,7 +386,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ C
           for (int i = 0; i < NC; ++i) v[i] = 0.f;
           const long long t0 = (long long)tile * p.kc;
           for (int ww = first; ww <= last; ++ww) {
-            const float* slot = p.partial + ((long long)(ww * 2 + (int)rank) * 2 + (Items::start(p, ww, W) >= t0 ? 0 : 1)) * SLOT_FLOATS;
+            const float* slot = p.partial + ((long long)(ww * 2 + (int)rank) * 2 + (Items::start(p, ww) >= t0 ? 0 : 1)) * SLOT_FLOATS;
 #pragma unroll
             for (int g = 0; g < NC / 8; ++g) {
               const float4* q = reinterpret_cast<const float4*>(slot + ((long long)(c / 8 + g) * TM + row_l) * 8);

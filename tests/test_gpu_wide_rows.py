@@ -99,13 +99,22 @@ def test_products_are_in_the_launch_timing(pair):
     assert nb.value == cfg.L * cfg.layer_matrix_bytes() + cfg.vocab * cfg.d_model * 2
 
 
+# deep rows (K = 8192 and more) beside few features, so that other products than the down product are split over K
+DEEP = {
+    "deep-qkv": dataclasses.replace(datagen.CONFIGS["8b"], name="deep-qkv", d_model=10240, n_q_heads=2, n_kv_heads=2, d_ffn=1280),
+    "deep-gate": dataclasses.replace(datagen.CONFIGS["8b"], name="deep-gate", d_model=8192, n_q_heads=16, n_kv_heads=2, d_ffn=3200),
+}
 # (model, rows, states): what the 74 pairs of CTAs do with the 256-row tiles of q/k/v, o, gate/up and down
 SCHEDULES = [
     ("mini8b", 1999, 1999),   # gate/up: 224 tiles, up to four per pair; nothing split (few chunks of K)
     ("mini8b", 1300, 26),     # gate/up: 168 tiles
     ("small", 1999, 1999),    # gate/up: 88 tiles on 74 pairs; q/k/v and o one per pair at most
-    ("8b", 129, 43),          # down: all 16 tiles split over 74 pairs; the others whole
-    ("8b", 1300, 260),        # down: 22 of 96 tiles split, then one whole tile per pair
+    ("8b", 129, 43),          # down: all 16 tiles split, four parts each; the others whole
+    ("8b", 257, 257),         # down: all 32 tiles split, two parts each
+    ("8b", 1300, 260),        # down: 22 of 96 tiles split, three parts each, then one whole tile per pair
+    ("8b", 1700, 340),        # down: 38 of 112 tiles split over all pairs: parts cross the tiles
+    ("deep-qkv", 1999, 1999), # q/k/v: all 24 tiles of the three matrices split; gate/up: 6 of 80, four parts each, then whole tiles
+    ("deep-gate", 700, 140),  # gate/up: one tile of 75 split, four parts
 ]
 
 
@@ -114,8 +123,8 @@ def test_schedules_of_the_products(model, rows, states):
     """Every row of a layer against the same rows in pieces of at most 128 (the persistent kernel, which the oracle checks at
     these shapes too), and three states against the oracle.  A bf16 operand is off by 2^-9 / sqrt(3) = 1.1e-3 (rms); each
     branch of the layer has two or three of those in a row, so a path is within about 3e-3 of the exact row and two paths
-    within 4e-3 of each other; twice that is allowed."""
-    cfg = dataclasses.replace(datagen.CONFIGS[model], L=1, vocab=64)
+    within 4e-3 of each other; twice that is allowed (the deep models, whose branches outweigh the residual stream, use most of it)."""
+    cfg = dataclasses.replace(DEEP.get(model) or datagen.CONFIGS[model], L=1, vocab=64)
     T, C = rows // states, 70
     p = Pair(cfg, max_ctx=C + T, max_rows=2048, max_M=1, max_T=1, gen_device="cuda")
     kv, ocache = p.new_kv(), p.new_oracle_cache()
