@@ -1458,7 +1458,7 @@ int clasp_dp_search(clasp_ctx* ctx, const float* hidden_states, int64_t layer_st
     if (first) {
       setup.first_rows = T; setup.first_d = d; setup.first_cell = M + 1;
       setup.x0 = hidden_states; setup.x1 = hidden_states + layer_stride; setup.x_stride = token_stride;
-      setup.g11 = ws.grow[1] + Td;
+      setup.g11 = ws.grow[1] + Td; setup.first_cos = ws.G; setup.first_done = &ws.ctl->first_done;
     }
     if ((rc = engine_launch(ctx, M * T, 0, setup, ctx_len))) return rc;
     clasp::backtrack_kernel<<<1, 256, 0, ctx->stream>>>(ws.choice, L, M, skip_mask);

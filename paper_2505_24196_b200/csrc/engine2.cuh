@@ -145,7 +145,8 @@ struct Bufs {
 struct Ctl {
   int abort;
   int status;
-  int pad[2];
+  int first_done;   // rows of a search's step 1 that the set-up kernel has done
+  int pad;
 };
 
 struct Job {

@@ -10,6 +10,7 @@ import pytest
 import torch
 
 import datagen
+import paper_2505_24196_b200 as clasp
 from oracle import clasp_oracle as orc
 from tests.util import Pair, check_search_against_oracle, kv_to_oracle, tol_hidden
 
@@ -88,3 +89,23 @@ def test_search_rows(pair, M, T):
     assert err.max() < tol_hidden(cfg), int(err.argmax())
     ok = ~np.isnan(ref["D"])
     np.testing.assert_allclose(rf["D"].cpu().numpy()[ok], ref["D"][ok], atol=1e-3)
+
+
+@pytest.mark.parametrize("T", [1, 2, 33, 128])
+def test_first_step_of_a_search(T):
+    """The one cell of step 1, the mean over the objective rows of cos(x_1, x_0), against float64, and again on the same
+    context (the rows' count has to be back at zero).  Sums of four fp32 products added in float64, then a handful of fp32
+    operations and the mean: within 1e-6."""
+    cfg = MINI
+    ccfg = clasp.make_config(cfg, max_ctx=160 + T, max_rows=128, max_M=1, max_T=T)
+    eng = clasp.Clasp(ccfg)
+    eng.load_layers(0, [datagen.layer_weights(cfg, l, "cuda") for l in range(cfg.L)])
+    kv = clasp.KVCache(ccfg)
+    for seed in (1, 2, 2):
+        g = torch.Generator(device="cuda").manual_seed(seed)
+        x = torch.randn((T, cfg.L + 1, cfg.d_model), device="cuda", generator=g).cumsum(1)
+        D = eng.dp_search(x, cfg.d_model, (cfg.L + 1) * cfg.d_model, kv, 160, 160, T, 1)["D"].cpu()
+        want = torch.nn.functional.cosine_similarity(x[:, 0].double(), x[:, 1].double(), dim=-1).mean()
+        assert D[1, 0] == 1.0 and abs(float(D[1, 1]) - float(want)) < 1e-6
+    assert eng.device_status() == 0
+    eng.close()
