@@ -975,6 +975,24 @@ int setup_launch(clasp_ctx* ctx, clasp::SetupArgs a) {
   return setup_launch_n<128>(ctx, a, bytes);
 }
 
+// Run length of a search's attention over `keys` cache positions: by the context and the head counts alone (not by its rows: a
+// row's sums must not depend on how many share the launch).  A kv head's runs and its own-key chunk are one chunk per CTA
+// where 16 runs (one trip of the merge) or 32 fit the grid.  Of more heads a CTA takes several chunks: as many runs, up to 16,
+// as need the fewest key tiles one after the other, a tile more per round of chunks for its start.  Searches of five layers, us,
+// 32 runs / only as many as are one chunk per CTA / as here: 64 kv heads of 64, 2000 positions 689 / 760 / 577, 3900 positions
+// 877 / 1143 / 790; 32 kv heads of 128, 2000 positions 584 / 572 / 534.
+int search_run_len(int keys, int n_kv_heads, int G) {
+  const int tiles = std::max(1, (keys + pk::ATT_KEYS - 1) / pk::ATT_KEYS), per_head = std::max(1, G / n_kv_heads - 1);
+  int runs = per_head >= 32 ? 32 : std::min(per_head, 16);
+  long best = 0;
+  for (int n = runs; per_head < 16 && n <= 16; ++n) {
+    const int len = (tiles + n - 1) / n;
+    const long chunks = (long)n_kv_heads * ((tiles + len - 1) / len + 1), cost = (chunks + G - 1) / G * (len + 1);
+    if (best == 0 || cost < best) { best = cost; runs = n; }
+  }
+  return pk::ATT_KEYS * ((tiles + runs - 1) / runs);
+}
+
 // Launch the engine over ctx->e_jobs.  Rmax: most rows of any job; head_off: first row of the
 // previous job that the head job (if any) reads.
 // `setup`: rotary table and the call's own tables or embedded rows; the rest of it is filled in here.
@@ -1098,15 +1116,8 @@ int engine_launch(clasp_ctx* ctx, int Rmax, int head_off, clasp::SetupArgs setup
   P.c.G = ctx->e_G; P.c.Rcap = ws.e_rcap; P.c.run_len = ws.e_run_len; P.c.chunk_cap = ws.e_chunk_cap;
   // The forward passes cut the cache into runs of a length fixed by the context capacity, so that a
   // position's attention is summed in the same order whichever call computes it (verification and
-  // one-token decoding must agree bit for bit).  The search only has to agree with itself: it cuts
-  // the keys it sees by the context and the head counts alone (not by its rows: a row's sums must not
-  // depend on how many share the launch) into so many runs that a kv head's runs and its own-key chunk are
-  // one chunk per CTA, and at most 16 where more do not fit (one trip of the merge).
-  if (search_ctx >= 0) {
-    const int per_head = std::max(1, ctx->e_G / c.n_kv_heads - 1);
-    const int runs = per_head >= 32 ? 32 : std::min(per_head, 16);
-    P.c.run_len = pk::ATT_KEYS * std::max(1, (search_ctx + pk::ATT_KEYS * runs - 1) / (pk::ATT_KEYS * runs));
-  }
+  // one-token decoding must agree bit for bit).  The search only has to agree with itself.
+  if (search_ctx >= 0) P.c.run_len = search_run_len(search_ctx, c.n_kv_heads, ctx->e_G);
   if (att_tc) {
     // run length: whole 64-key tiles, at most 32 runs; the cut that needs the fewest tile steps when the
     // (kv head, run, pair block) items are dealt out to the CTAs (one more step per round for its set-up)

@@ -12,7 +12,7 @@ import torch
 import datagen
 import paper_2505_24196_b200 as clasp
 from oracle import clasp_oracle as orc
-from tests.util import Pair, check_search_against_oracle, kv_to_oracle, tol_hidden
+from tests.util import Pair, check_search_against_oracle, kv_to_oracle, scaled_keys, search_that_applies_layer_1, tol_hidden
 
 pytestmark = pytest.mark.gpu
 MINI = datagen.CONFIGS["mini8b"]
@@ -109,3 +109,26 @@ def test_first_step_of_a_search(T):
         assert D[1, 0] == 1.0 and abs(float(D[1, 1]) - float(want)) < 1e-6
     assert eng.device_status() == 0
     eng.close()
+
+
+@pytest.mark.parametrize("nq,nkv,hd,C,T", [
+    (32, 32, 128, 200, 3),     # a run of the context per CTA
+    (32, 32, 128, 2400, 3),    # eight or so runs per kv head: a CTA takes chunks of several heads
+    (64, 64, 64, 1000, 40),
+    (64, 64, 64, 2400, 3),
+    (64, 16, 64, 2400, 40),    # 160 (row, query head) pairs per kv head: the form that walks consecutive chunks
+    (33, 33, 128, 700, 2),     # a number of heads that does not divide the grid
+])
+def test_search_with_many_kv_heads(nq, nkv, hd, C, T):
+    """More kv heads than leave the grid 16 chunks each: the runs of a search's attention are cut by rounds of chunks.  The search's
+    best state is a layer output it computed, compared row by row with the oracle (keys scaled so that every tile counts)."""
+    cfg = dataclasses.replace(MINI, name="heads", L=2, n_q_heads=nq, n_kv_heads=nkv, head_dim=hd, d_ffn=512, vocab=64)
+    m = Pair(cfg, max_ctx=C, max_rows=64, max_M=1, max_T=T, gen_device="cuda")
+    m.kv, m.ocache = m.new_kv(), m.new_oracle_cache()
+    for t, k in ((m.kv.k, 0), (m.kv.v, 1)):
+        t.copy_(datagen.normal_rows(83, k, tuple(t.shape)).to(cfg.torch_dtype))
+    kv_to_oracle(m.kv, C, m.ocache)
+    assert m.engine.engine_active()
+    with scaled_keys(m, 0, 4):
+        search_that_applies_layer_1(m, C, T, 84)
+    m.engine.close()
