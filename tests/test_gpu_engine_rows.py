@@ -12,7 +12,8 @@ import torch
 import datagen
 import paper_2505_24196_b200 as clasp
 from oracle import clasp_oracle as orc
-from tests.util import Pair, check_search_against_oracle, kv_to_oracle, scaled_keys, search_that_applies_layer_1, tol_hidden
+from tests.util import (Pair, check_search_against_oracle, kv_to_oracle, rel_l2, scaled_keys, search_that_applies_layer_1,
+                        tol_hidden)
 
 pytestmark = pytest.mark.gpu
 MINI = datagen.CONFIGS["mini8b"]
@@ -132,3 +133,81 @@ def test_search_with_many_kv_heads(nq, nkv, hd, C, T):
     with scaled_keys(m, 0, 4):
         search_that_applies_layer_1(m, C, T, 84)
     m.engine.close()
+
+
+FORWARDS = {
+    "slices-of-8": MINI,
+    "hd64": datagen.CONFIGS["small"],
+    "slices-of-32": dataclasses.replace(datagen.CONFIGS["8b"], name="8b-l2", vocab=4096, L=2),
+    # slices past 64 features: a lane quarter of the accumulator holds 32 of them instead of 16; eight query heads per kv head
+    "slices-of-72": dataclasses.replace(MINI, name="wider-slice", d_model=10240, n_q_heads=16, n_kv_heads=2, d_ffn=512, vocab=2048, L=2),
+}
+
+
+@pytest.mark.parametrize("model", list(FORWARDS))
+@pytest.mark.parametrize("n,C", [(40, 517), (64, 100)])   # (from 65 rows on the CTAs start their walks over K elsewhere)
+def test_forward_rows_do_not_depend_on_the_rows_of_the_call(model, n, C):
+    """The same tokens in one call, whose (row, query head) pairs need several blocks of 128, and in calls of at most one
+    block: states, keys, values and logits are the same bits (verification, of 64 rows at most, and one-token decoding must
+    agree)."""
+    cfg, K = FORWARDS[model], 7
+    per_call = 128 // (cfg.n_q_heads // cfg.n_kv_heads)
+    assert n > per_call > K
+    ccfg = clasp.make_config(cfg, max_ctx=MAX_CTX, max_rows=128, max_M=1, max_T=1)
+    eng = clasp.Clasp(ccfg)
+    eng.load_layers(0, [datagen.layer_weights(cfg, l, "cuda") for l in range(cfg.L)])
+    eng.load_head(datagen.head_weights(cfg, "cuda"))
+    g = torch.Generator(device="cuda").manual_seed(17)
+    toks = torch.randint(0, cfg.vocab, (n,), device="cuda", dtype=torch.int32, generator=g)
+    q = torch.zeros((K, cfg.vocab), device="cuda")
+    k0, v0 = (torch.randn((cfg.L, C, cfg.n_kv_heads, cfg.head_dim), device="cuda", generator=g).to(torch.bfloat16) for _ in range(2))
+
+    def call(pieces):
+        kv = clasp.KVCache(ccfg)
+        kv.k[:, :C], kv.v[:, :C] = k0, v0
+        hidden, lo = [], 0
+        for m in pieces[:-1]:
+            hidden.append(eng.verify(toks[lo:lo + m].clone(), C + lo, kv, 0)[1])
+            lo += m
+        hidden.append(torch.empty((n - lo, cfg.L + 1, cfg.d_model), device="cuda"))
+        p = torch.empty((K + 1, cfg.vocab), device="cuda")
+        out = torch.zeros(1, dtype=torch.int32, device="cuda"), torch.zeros(K + 1, dtype=torch.int32, device="cuda")
+        eng.verify_sample(toks[lo:].clone(), C + lo, kv, K, q, 1.0, 5, 1, p, *out, hidden[-1])
+        return {"hidden": torch.cat(hidden), "k": kv.k[:, C:C + n], "v": kv.v[:, C:C + n], "logits": p}
+
+    whole = call([n])
+    rest = n - (K + 1)
+    cuts = [min(per_call, rest - lo) for lo in range(0, rest, per_call)]
+    some = call(cuts + [K + 1])
+    assert eng.device_status() == 0
+    for key in whole:
+        assert torch.equal(whole[key], some[key]), key
+    eng.close()
+
+
+@pytest.mark.parametrize("L", [98, 99, 101])
+def test_models_of_many_layers(L):
+    """The job list travels as a kernel parameter up to 99 jobs and is copied beyond: a verification has L + 1 jobs, a search
+    L - 1.  Against the oracle, whose decisions the search is given."""
+    cfg = dataclasses.replace(MINI, name="deep", L=L, d_model=128, n_q_heads=2, n_kv_heads=1, head_dim=64, d_ffn=128, vocab=64)
+    n, T, M = 12, 2, 2
+    p = Pair(cfg, max_ctx=32, max_rows=64, max_M=M, max_T=T)
+    toks = datagen.token_ids(cfg, n)
+    ocache, kv = p.new_oracle_cache(), p.new_kv()
+    _, hid_o, _ = orc.verify_forward(p.oracle, toks.numpy(), ocache, 0)
+    _, hid = p.engine.verify(toks.cuda(), 0, kv, n)
+    assert p.engine.engine_active()
+    assert rel_l2(hid.cpu().numpy(), hid_o) < tol_hidden(cfg)
+    x_o, p0 = np.transpose(hid_o[n - T:], (1, 0, 2)), n - T
+    kv.k.copy_(torch.from_numpy(ocache.k).to(cfg.torch_dtype))
+    kv.v.copy_(torch.from_numpy(ocache.v).to(cfg.torch_dtype))
+    ref = orc.dp_search(p.oracle, x_o, ocache, p0, p0, M)
+    x = torch.from_numpy(np.ascontiguousarray(hid_o[n - T:])).float().cuda()
+    res = p.engine.dp_search(x, cfg.d_model, (L + 1) * cfg.d_model, kv, p0, p0, T, M,
+                             forced_choice=torch.from_numpy(ref["choice"].copy()).cuda())
+    D = res["D"].cpu().numpy()
+    assert np.array_equal(np.isnan(D), np.isnan(ref["D"]))
+    np.testing.assert_allclose(D[~np.isnan(D)], ref["D"][~np.isnan(D)], atol=1e-3)
+    assert np.array_equal(res["S"].cpu().numpy(), ref["S"])
+    assert p.engine.device_status() == 0
+    p.engine.close()
