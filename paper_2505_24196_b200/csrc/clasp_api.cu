@@ -209,7 +209,7 @@ struct clasp_ctx {
   int e_G = 0;              // CTAs of the cooperative grid (one per SM)
   int e_static_smem = 0;
   const void* e_kernel[2 * clasp::pk::N_KINDS] = {};   // the layer kernel for this head dimension by kind, plain and with step stamps
-  int e_split_lo[clasp::pk::N_SPLITS], e_split_units[clasp::pk::N_SPLITS], e_tile_idx[5], e_tiles_off = 0,
+  int e_split_lo[clasp::pk::N_SPLITS], e_tile_idx[5], e_tiles_off = 0,
       e_kpi[5], e_use3d[5], e_wpages[5];
   int e_heights[8][clasp::pk::N_HEIGHTS];   // tile heights per matrix slot (wq wk wv wo gate up down head)
   std::vector<CUtensorMap> e_wmaps_host;
@@ -864,7 +864,6 @@ int engine_setup(clasp_ctx* ctx) {
       for (int cc = 0; cc <= G; ++cc) lo[s][cc] = (int)(units * cc / G) * 8;
     }
     ctx->e_split_lo[s] = (int)tab.size();
-    ctx->e_split_units[s] = split_n[s] / 8;
     tab.insert(tab.end(), lo[s].begin(), lo[s].end());
   }
   for (int cc = 0; cc < G; ++cc)
@@ -1031,7 +1030,10 @@ int engine_launch(clasp_ctx* ctx, int Rmax, int head_off, clasp::SetupArgs setup
   // an item (gate + up rows and the operand tiles of kpi chunks) must fit the ring twice over
   const int b_pages = BN * pk::BK * 2 / pk::PAGE;
   // chunks per ring item in this launch: the set-up value when two such items fit the ring, else fewer,
-  // loaded chunk by chunk through the 2-D maps (the 3-D boxes are built for the set-up value)
+  // loaded chunk by chunk through the 2-D maps (the 3-D boxes are built for the set-up value).  Up to 64 rows (48 of a search
+  // that hands both candidates on, on the 8B shape) it is the set-up value.  With more a CTA starts its walk over K at another
+  // chunk, so a row's sums are then added in another order.  (A start in units of the set-up's items and a ragged item at the
+  // seam make them the same bits for any number of rows, at 1.3 % of the 8B search and 1.8 % of a 128-row prefill.)
   bool any_dual = false;
   for (const pk::Job& J : ctx->e_jobs) any_dual = any_dual || J.dual_src;
   int kpi[5], use3d[5];
@@ -1133,9 +1135,9 @@ int engine_launch(clasp_ctx* ctx, int Rmax, int head_off, clasp::SetupArgs setup
     }
     P.c.run_len = best_len;
   }
-  P.c.BN = BN; P.c.ring_pages = ring_pages; P.c.stage_bytes = BN * n_slice * 4; P.c.att_tc = att_tc ? 1 : 0; P.c.att_rows = att_rows;
+  P.c.BN = BN; P.c.ring_pages = ring_pages; P.c.stage_bytes = BN * n_slice * 4; P.c.att_rows = att_rows;
 
-  for (int s = 0; s < pk::N_SPLITS; ++s) { P.c.split_lo[s] = ctx->e_split_lo[s]; P.c.split_units[s] = ctx->e_split_units[s]; }
+  for (int s = 0; s < pk::N_SPLITS; ++s) P.c.split_lo[s] = ctx->e_split_lo[s];
   for (int k = 0; k < 5; ++k) { P.c.tile_idx[k] = ctx->e_tile_idx[k]; P.c.kpi[k] = kpi[k]; P.c.use3d[k] = use3d[k]; }
   P.c.tiles_off = ctx->e_tiles_off; P.c.map3d_off = (int)(((size_t)c.L * 7 + 1) * pk::N_HEIGHTS);
   P.b.xn_a = (bf16*)ws.xn; P.b.xn_m = (bf16*)ws.xn_m; P.b.attn = (bf16*)ws.attn; P.b.act = (bf16*)ws.act;

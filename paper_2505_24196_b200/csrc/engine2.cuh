@@ -110,11 +110,8 @@ struct Cfg {
   int ring_pages;
   int stage_bytes;     // worker scratch taken by the slices of the launch's rows in an epilogue (the per-row floats follow)
   int att_rows;        // tensor-core attention: (row, query head) pairs per item, 64 or 128
-  int att_tc;          // 1: search jobs run the attention over their cache keys on tcgen05 (kernel instantiation with
-                       // TC set; the launch carries SCRATCH_TC_BYTES of worker scratch instead of SCRATCH_BYTES)
   // tables (ints / structs in Params::tabs, offsets in ints)
   int split_lo[N_SPLITS];    // [G + 1] first feature of each CTA: lo(c) = 8 floor(c units / G)
-  int split_units[N_SPLITS]; // 8-feature units of each split
   int tile_idx[5];           // per product kind: [G + 1] first TileDesc of each CTA
   int tiles_off;             // TileDesc array
   int kpi[5];                // 64-column chunks per ring item
@@ -223,9 +220,6 @@ __device__ __forceinline__ int ld_acquire_i32(const int* p) {
   int v;
   asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
-}
-__device__ __forceinline__ void st_release_i32(int* p, int v) {
-  asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 __device__ __forceinline__ int ld_volatile_i32(const int* p) {
   int v;
@@ -362,7 +356,6 @@ struct Shared {
   uint32_t wait_fast, wait_slow;   // the launch's wait limits
   volatile int a_issued;    // ring items whose weight loads have been issued (warp 0 -> warp 1)
   int b_seen;               // products whose operand warp 1 has seen complete (warp 1 -> workers)
-  int flag;                 // broadcast of a one-thread decision to the workers
   float rs[MAX_ROWS];       // per-row norm factors of the current product
   float rs_next[MAX_ROWS];  // Eq. 2 step: norm factors of the rows it hands to the next layer
   int choice_row[MAX_ROWS + 16];  // Eq. 2 decision per candidate row (1: the layer output was taken)
@@ -822,12 +815,6 @@ struct Worker {
     if (wtid == 0) ok = wait_count(p, kind, tgt, sh);
     return worker_and(ok);
   }
-  // wait for flags [first, first + n) of `kind`: one flag per thread
-  __device__ bool wait_flags(int kind, int first, int n, int epoch) {
-    bool ok = true;
-    for (int k = wtid; k < n; k += WORKERS) ok = wait_flag(p.b.flags + kind * p.c.G + first + k, epoch, p.ctl, sh) && ok;
-    return worker_and(ok);
-  }
 
   // Feature (row of an accumulator of n rows) that thread `lane` of lane quarter `quarter` owns, or -1:
   // an M = 128 accumulator has row r in lane r, an M = 64 one (n <= 64) in lane 32 (r / 16) + r % 16.
@@ -866,16 +853,10 @@ struct Worker {
   // RB accumulator columns of this thread's lane
   __device__ __forceinline__ static void tmem_ld_rb(uint32_t taddr, float (&v)[RB]) {
     uint32_t r[RB];
-    if constexpr (RB == 8) {
-      asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                   : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                   : "r"(taddr));
-    } else {
-      static_assert(RB == 4 || RB == 8, "row block of 4 or 8 accumulator columns");
-      asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
-                   : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-                   : "r"(taddr));
-    }
+    static_assert(RB == 4, "row block of 4 accumulator columns");
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(taddr));
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
     for (int i = 0; i < RB; ++i) v[i] = __uint_as_float(r[i]);
@@ -2736,7 +2717,6 @@ engine_kernel(const __grid_constant__ CUtensorMap map_xn_a, const __grid_constan
     sh.wait_slow = p.wait_slow;
     sh.a_issued = 0;
     sh.b_seen = 0;
-    sh.flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
