@@ -348,8 +348,8 @@ int64_t clasp_launch_count(const clasp_ctx* ctx);
  * paper).  `stamps` is DEVICE memory of n_ctas * cap_per_cta uint64 (borrowed until it is
  * replaced or cleared with NULL): during every following search / verify / draft call the
  * kernel's CTA c writes %globaltimer values (ns) to stamps[c * cap_per_cta + 64 * j + s]
- * when it reaches step boundary s of job j of the call (jobs: one per decoder layer pass or
- * Eq. 2 step, then the LM head; s: 0 job start, 1 q/k/v done, 2-5 attention partials, 6
+ * when it reaches step boundary s of job j of the call (jobs: one per decoder layer pass, then the
+ * LM head; of a search one per Eq. 2 step from step 2 on, step 1 being done ahead of them; s: 0 job start, 1 q/k/v done, 2-5 attention partials, 6
  * attention merged, 7 o, 8 gate/up, 9 down, 10-13 Eq. 2 step, 14 head; for product p = 0..3
  * (q/k/v, o, gate/up, down) 16+p first operands ready for the tensor core, 20+p last
  * multiply issued, 24+p first accumulator complete; 28 Eq. 2 step published the next operand;

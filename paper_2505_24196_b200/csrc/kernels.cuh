@@ -656,8 +656,8 @@ __global__ void __launch_bounds__(256) setup_kernel(const __grid_constant__ Setu
   }
   if (a.first_rows > 0) {
     // a block per row, from the middle of the grid on (blocks with little else to do); the block that comes last adds the rows'
-    // cosines in row order.  (One block for all rows took 2.2 us a
-    // row: searches of four layers of the 8B shape, M = 1, T = 8 / 64 / 128: 339 / 555 / 942 -> 330 / 458 / 663 us.)
+    // cosines in row order.  (One block for all rows took 2.2 us a row: searches of four layers of the 8B shape, M = 1, T = 8 /
+    // 64 / 128: 339 / 555 / 942 -> 330 / 458 / 663 us.)
     __shared__ double part[3][8];
     __shared__ float cosines[256];
     __shared__ bool last;

@@ -226,9 +226,10 @@ __device__ __forceinline__ bool epi_any(bool p) {
 // both, each keeps the accumulator of its own 128 rows.  A 64-column chunk is 512 cycles of multiplies for 32 KB of loads
 // per SM (one CTA per tile of 128 x 256 would need 48 KB for the same work).  Measured, 8B shape, 1999 rows, PFLOP/s in a
 // loop under the power cap, a plain library product of the same shape beside it: gate/up 1.22 / 1.25, q/k/v 1.06 / 1.27, o
-// 0.94 / 1.28, down 1.11 / 1.32.  All four read about 11 TB/s from L2 into shared memory; gate/up is at the power cap beside.
-// (Passes of 256 rows through the skinny product, which re-read all weights eight times, and the CUDA-core attention took
-// 14.9 ms per layer together.)  At
+// 0.94 / 1.28, down 1.11 / 1.32.  Gate/up is at the power cap.  The others have two or three waves of tiles (o and down 1.7 of
+// 2, q/k/v 2.6 of 3); their loads, 64 KB per pair and chunk, come to 11.6 TB/s for gate/up and 9.0, 7.9 and 9.7 for q/k/v, o
+// and down, so the rate of L2 does not bound them, and what takes the rest is not known.  (Passes of 256 rows through the
+// skinny product, which re-read all weights eight times, and the CUDA-core attention took 14.9 ms per layer together.)  At
 // 128 rows the four products take 216 us against 114 inside the persistent kernel (partial sums, ramps), so that kernel
 // keeps the launches of up to 128 rows.
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS, 1)
